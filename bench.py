@@ -571,6 +571,23 @@ def run_gpu(args, rank, world, local):
         if prec_info:
             line["precision"] = prec_info
             line["roofline"]["traffic"] = None
+        delayed = stats[0]["path"] == 1 and args.layout == "condensed"
+        if delayed:
+            line["roofline"]["kernel"] = "k_pivot_delayed"
+            line["roofline"]["what"] = ("bytes the pivots' update passes and side reads move (several pivots per "
+                                        "pass over the tableau)")
+        if delayed and args.precision == "fp64":
+            # several pivots per pass over the tableau: the FP64 pipe is the
+            # ceiling (one fma per condensed entry and pivot), not HBM
+            peak_f, probe = fp64_fma_rate(tsx, sptr)
+            flops = 2.0 * (m + 1) * (n + 1) * pivots / args.steps
+            ach = flops / (kernel_ms / 1000.0) / 1e12
+            line["roofline"].update({
+                "bound": "alu", "achieved": ach, "peak": peak_f, "unit": "TFLOP/s", "frac": ach / peak_f,
+                "peak_source": "measured FP64 fma rate in this run (lp_measure_fp64_fma_rate)",
+                "probe": probe, "flops_per_launch": flops,
+                "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+                        "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)"}})
         if stats[0]["path"] == 4:
             # the cluster path keeps the tableau on chip: its ceiling is the
             # FP64 pipes of the cluster's SMs, not HBM

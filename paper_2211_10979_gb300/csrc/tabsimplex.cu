@@ -102,6 +102,12 @@ struct Work {                        // pivot buffers for one precision and layo
     int* act = nullptr;
     ArgPart* cpart = nullptr;
     RatPart* rpart = nullptr;
+    // condensed: buffers of the delayed updates (tsx_delayed.cuh)
+    void* Fh = nullptr;
+    void* Rh = nullptr;
+    void* RhT = nullptr;
+    void* rhs = nullptr;
+    DelayRec* recs = nullptr;        // 2 x max_grid
 };
 
 struct RecBufs {                     // FP64 recovery buffers
@@ -592,6 +598,12 @@ static lp_status ensure_work(lp_handle* h, int elem, int cond) {
     const size_t o_cp = cv.take((size_t)nstrips * sizeof(ArgPart));
     const size_t o_rp = cv.take((size_t)h->max_grid * sizeof(RatPart));
     const size_t o_var = cv.take((size_t)h->n * sizeof(int));
+    const size_t K = cond ? (elem == 8 ? DelayK<double>::K : DelayK<float>::K) : 0;
+    const size_t o_Fh = cv.take((size_t)(h->m + 1) * K * elem);
+    const size_t o_Rh = cv.take((size_t)ld * K * elem);
+    const size_t o_RhT = cv.take((size_t)ld * K * elem);
+    const size_t o_rhs = cv.take(cond ? (size_t)(h->m + 1) * elem : 0);
+    const size_t o_recs = cv.take(cond ? 2 * (size_t)h->max_grid * sizeof(DelayRec) : 0);
     if (!dev_alloc_block(h, h->work.blk, align_up(cv.off, 256))) {
         set_error("lp_solve: device allocation of %zu bytes for the tableau failed", cv.off);
         return LP_ERR_NOMEM;
@@ -608,6 +620,13 @@ static lp_status ensure_work(lp_handle* h, int elem, int cond) {
     h->work.act = (int*)(base + o_act);
     h->work.cpart = (ArgPart*)(base + o_cp);
     h->work.rpart = (RatPart*)(base + o_rp);
+    if (cond) {
+        h->work.Fh = base + o_Fh;
+        h->work.Rh = base + o_Rh;
+        h->work.RhT = base + o_RhT;
+        h->work.rhs = base + o_rhs;
+        h->work.recs = (DelayRec*)(base + o_recs);
+    }
     return LP_OPTIMAL;
 }
 
@@ -660,6 +679,84 @@ static int max_coresident(int device) {
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pivot_persistent<NT, V>, NT, persistent_smem<NT>());
     return nsm * per;
+}
+
+// ------------------------------------------------------- delayed updates
+// Dynamic shared memory of a block of k_pivot_delayed: the staging of a pass
+// and, where the limit `limit` allows, the block's own parts of the LP.
+template <int NT, typename V>
+static size_t delayed_smem(int m, int n, int blocks, size_t limit) {
+    const size_t pass = delay_smem_bytes<V>(NT, delayed_rows(NT));
+    const size_t own = delay_own_bytes<V>(m, n, blocks, pass);
+    return own <= limit ? own : pass;
+}
+
+// Blocks of NT threads of k_pivot_delayed that fit the device together, and
+// the dynamic shared memory each of them may use.
+template <int NT, typename V>
+static int delayed_coresident(int device, size_t& smem_limit) {
+    constexpr int want = persistent_sm_threads(NT) / NT;   // blocks per SM the kernel is built for
+    static std::once_flag once;
+    static size_t limit = 0;
+    std::call_once(once, [device] {
+        int per_sm = 0, reserved = 0, optin = 0;
+        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device);
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, k_pivot_delayed<NT, V>) == cudaSuccess) {
+            const long long lim = std::min((long long)per_sm / want - reserved, (long long)optin) -
+                                  (long long)fa.sharedSizeBytes;
+            if (lim > 0 && cudaFuncSetAttribute((const void*)k_pivot_delayed<NT, V>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim) == cudaSuccess)
+                limit = (size_t)lim;
+        }
+        cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+    });
+    smem_limit = limit;
+    if (limit < delay_smem_bytes<V>(NT, delayed_rows(NT))) return 0;
+    int nsm = 0, per = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pivot_delayed<NT, V>, NT, limit) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return nsm * per;
+}
+
+template <typename V>
+static Delayed<V> delayed_params(lp_handle* h, const lp_options& o, double eps_d, double eps_p) {
+    Delayed<V> D{};
+    D.T = (V*)h->work.T;
+    D.ld = h->work.ld;
+    D.m = h->m;
+    D.n = h->n;
+    D.basis = h->basis;
+    D.var = h->work.var;
+    D.Fh = (V*)h->work.Fh;
+    D.Rh = (V*)h->work.Rh;
+    D.RhT = (V*)h->work.RhT;
+    D.rhs = (V*)h->work.rhs;
+    D.rat = h->work.recs;
+    D.arg = h->work.recs + h->max_grid;
+    D.bar_count = &h->st->bar_count;
+    D.fail = &h->st->fail;
+    D.status = &h->st->status;
+    D.eps_d = eps_d;
+    D.eps_p = eps_p;
+    D.max_iters = o.max_iters < 0 ? 50LL * ((long long)h->m + h->n) : o.max_iters;
+    D.k_cyc = o.k_cyc;
+    D.rule = o.rule;
+    D.timeout_ns = std::max(0LL, o.barrier_timeout_ns);
+    return D;
+}
+
+// Blocks of a delayed solve: all that fit, fewer for LPs with less than four
+// rows and columns a block.
+static int delayed_grid(int m, int n, int resident, int max_grid, int user_blocks) {
+    int g = std::min(std::min(resident, max_grid), std::max(1, (std::max(m + 1, n) + 3) / 4));
+    if (user_blocks > 0) g = std::min(g, user_blocks);
+    return std::max(1, g);
 }
 
 template <int NT, typename V>
@@ -996,7 +1093,7 @@ static lp_status run_hybrid(lp_handle* h, const lp_options& o, cudaStream_t s, c
 // Runs the pivot phase (build + Steps 1-3) on the handle's tableau of V.
 template <int NT, typename V>
 static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, double eps_d, double eps_p,
-                             DevState& hs, long long& launches, int& path_used, int& grid_used) {
+                             DevState& hs, long long& launches, int& path_used, int& grid_used, bool& delayed) {
     const int m = h->m, n = h->n;
     const int ld = h->work.ld;
     Params<V> P = make_params<V>(m, n, ld, (V*)h->work.T, (V*)h->work.F, (V*)h->work.R, h->work.act,
@@ -1035,6 +1132,16 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     }
 
     // Initialization Step
+    // the condensed tableau's persistent path delays its updates
+    int dgrid = 0;
+    size_t dsmem = 0;
+    if (path == LP_PATH_PERSISTENT && h->work.cond && !TSX_TMA) {
+        const int resident = delayed_coresident<NT, V>(h->device, dsmem);
+        if (resident > 0) {
+            dgrid = delayed_grid(m, n, resident, h->max_grid, o.blocks);
+            dsmem = delayed_smem<NT, V>(m, n, dgrid, dsmem);
+        }
+    }
     cudaEventRecord(h->ev[0], s);
     k_reset_state<<<1, 32, 0, s>>>(h->st);
     {
@@ -1081,7 +1188,20 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
         grid_run = csize;
     }
     if (path == LP_PATH_PERSISTENT) {
-        cudaError_t e = launch_persistent<NT, V>(P, grid, s);
+        cudaError_t e = cudaSuccess;
+        if (dgrid) {
+            Delayed<V> D = delayed_params<V>(h, o, eps_d, eps_p);
+            D.smem = (unsigned)dsmem;
+            D.qlog = P.qlog;
+            D.plog = P.plog;
+            D.log_cap = P.log_cap;
+            DevState* st = h->st;
+            void* args[] = {(void*)&D, (void*)&st};
+            grid_run = dgrid;
+            e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
+        } else {
+            e = launch_persistent<NT, V>(P, grid, s);
+        }
         if (e != cudaSuccess) {
             if (o.path == LP_PATH_AUTO) {   // co-residency refused: fall back
                 cudaGetLastError();
@@ -1103,6 +1223,7 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     CUDA_TRY(cudaStreamSynchronize(s), LP_ERR_CUDA);
     path_used = path;
     grid_used = grid_run;
+    delayed = dgrid > 0 && path == LP_PATH_PERSISTENT;
     if (hs.status == kRunning) {
         set_error("lp_solve: kernel ended without a status");
         return LP_ERR_CUDA;
@@ -1432,10 +1553,11 @@ static lp_status solve_nt(lp_handle* h, const lp_options& o, cudaStream_t s) {
     DevState hs{};
     long long launches = 0;
     int path = 0, grid = 0;
+    bool delayed = false;
     if (fp32)
-        st = pivot_phase<NT, float>(h, o, s, o.eps_d_fp32, o.eps_p_fp32, hs, launches, path, grid);
+        st = pivot_phase<NT, float>(h, o, s, o.eps_d_fp32, o.eps_p_fp32, hs, launches, path, grid, delayed);
     else
-        st = pivot_phase<NT, double>(h, o, s, o.eps_d, o.eps_p, hs, launches, path, grid);
+        st = pivot_phase<NT, double>(h, o, s, o.eps_d, o.eps_p, hs, launches, path, grid, delayed);
     if (st == LP_ERR_CUDA) return st;
 
     float ms_build = 0.f, ms_pivot = 0.f;
@@ -1450,7 +1572,14 @@ static lp_status solve_nt(lp_handle* h, const lp_options& o, cudaStream_t s) {
     // 1..m except p, read + write of the objective row and write of row p over
     // all groups; plus the side traffic of Steps 1-2 and the staging: column q
     // and right-hand-side sectors (m + 1 rows), pivot row read, R write + read.
-    {
+    // Delayed updates: a read and a write of rows 1..m per pass, and per pivot
+    // the sectors of column q (read, and set to zero) and row p, the row
+    // entries and multipliers stored for the pass.
+    if (delayed) {
+        const double pass = 64.0 * (double)m * (double)((h->n + E - 1) / E);
+        const double side = 96.0 * (double)(m + 1) + 4.0 * elem * (double)ld;
+        h->stats.update_bytes = pass * (double)hs.passes + side * (double)hs.iters;
+    } else {
         const double nsec = (double)(ld / E);
         const double upd = 64.0 * (double)(m - 1) * (double)hs.active_sectors + 96.0 * nsec * (double)hs.iters;
         const double side = (64.0 * (double)(m + 1) + 3.0 * elem * (double)ld) * (double)hs.iters;

@@ -118,6 +118,8 @@ struct DevState {
     int qvar;                          // entering variable (one-launch-per-phase path)
     unsigned nact;                     // active 32-B column groups of this pivot
     unsigned next_slot;                // P4 work counter (slots handed out)
+    int fail;                          // delayed updates: a wait ran out
+    unsigned passes;                   // delayed updates: passes over the tableau
     long long phase_ns[6];             // block 0's time per phase: work of
                                        // {select+ratio, stage, update}, then the
                                        // barrier wait after each of them

@@ -6,12 +6,15 @@
 //                         host link, copied and checked in one pass
 //   k_build<V>            Initialization Step: Table I tableau (full or
 //                         condensed), slack basis
-//   k_pivot_persistent    Steps 1-3 iterated inside one cooperative launch
+//   k_pivot_delayed       Steps 1-3 iterated inside one cooperative launch on a
+//                         condensed tableau, updates delayed (tsx_delayed.cuh)
+//   k_pivot_persistent    the same with one update per pivot (the full layout)
 //   k_ml_*                the same phases, one launch each (fallback, profiling)
 //   k_extract_*<V>        read-out of x, y, objective from the tableau
 //   k_expand_cond<V> etc. Table I rebuilt from a condensed tableau
 #pragma once
 
+#include "tsx_delayed.cuh"
 #include "tsx_device.cuh"
 
 namespace tsx {
@@ -31,6 +34,8 @@ __global__ void k_reset_state(DevState* st) {
         st->bar_gen = 0;
         st->nact = 0;
         st->next_slot = 0;
+        st->fail = 0;
+        st->passes = 0;
         for (int k = 0; k < 6; ++k) st->phase_ns[k] = 0;
     }
 }
@@ -275,6 +280,36 @@ __global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_pe
         clk.lap(2);
         if (!pivot_barrier(P.st, P.timeout_ns, s)) return;
         clk.lap(5);
+    }
+}
+
+// The condensed tableau's persistent kernel: one cooperative launch, the grid's
+// blocks as the blocks of one delayed solve.
+// Rows of an update tile: two tiles of 8 rows fill half of 255 registers.
+__host__ __device__ constexpr int delayed_rows(int nt) { return persistent_sm_threads(nt) <= 256 ? 8 : 4; }
+template <int NT, typename V>
+__global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_delayed(Delayed<V> lp, DevState* st) {
+    extern __shared__ __align__(128) unsigned char tsx_dyn[];
+    __shared__ DelayScratch s;
+    __shared__ DelayState S;
+    __shared__ PhaseClock clk;
+    __shared__ Delayed<V> D;
+    if (threadIdx.x == 0) {
+        D = lp;
+        D.bt = blockIdx.x;
+        D.G = gridDim.x;
+        s.passed = 0;
+    }
+    __syncthreads();
+    clk.start();
+    delayed_solve<NT, delayed_rows(NT)>(D, tsx_dyn, s, S, clk);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && S.status != kDelayFailed) {
+        atomicCAS(&st->status, kRunning, S.status);
+        st->iters = S.it;
+        st->bland = S.bland;
+        st->degen_run = S.degen;
+        st->passes = S.passes;
+        for (int k = 0; k < 6; ++k) st->phase_ns[k] = clk.acc[k];
     }
 }
 

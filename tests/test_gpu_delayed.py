@@ -1,0 +1,79 @@
+"""Delayed updates (the condensed tableau's persistent path): up to 16 (FP32:
+32) pivots share one pass over the tableau.
+
+Every entry takes the undelayed update's fused multiply-adds in the same order,
+so the tableau, the pivots and the results equal the oracle's, and where entries
+overflow the undelayed condensed path's, entry for entry (tolerance 0).
+"""
+import numpy as np
+import pytest
+
+import lpgen
+import oracle
+
+from test_gpu_parity import _assert_same, _gpu_run, _oracle_run, tsx  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+# columns around a strip (128 doubles, 256 floats) and a 32-byte group, rows
+# around a tile (8); pivots around a round (16, 32); and one block, whose own
+# rows and columns do not fit its shared memory
+SHAPES = [(8, 127), (9, 128), (7, 129), (255, 257), (63, 1021)]
+
+
+@pytest.mark.parametrize("m,n", SHAPES)
+@pytest.mark.parametrize("k", [1, 15, 16, 17, 33, -1])
+def test_rounds_and_remainders(tsx, m, n, k):   # noqa: F811
+    A, b, c = lpgen.diag_dominant_lp(m, n, 3 + m)   # about min(m, n) pivots or more
+    ref = _oracle_run(A, b, c, max_iters=k)
+    _assert_same(_gpu_run(tsx, A, b, c, path=1, max_iters=k), ref)
+
+
+@pytest.mark.parametrize("m,n", [(9, 255), (40, 257), (257, 300)])
+def test_float_rounds(tsx, m, n):   # noqa: F811
+    A, b, c = lpgen.diag_dominant_lp(m, n, 5 + m)
+    st32, it32, qref, pref, Tref, _ = oracle.solve32(A, b, c)
+    _, _, T, q, p, stats = _gpu_run(tsx, A, b, c, path=1, precision=tsx.LP_PREC_FP32)
+    assert stats["pivot_status"] == st32 and stats["iters"] == it32
+    np.testing.assert_array_equal(q, qref)
+    np.testing.assert_array_equal(p, pref)
+    np.testing.assert_array_equal(T, Tref.astype(np.float64))
+
+
+@pytest.mark.parametrize("blocks", [1, 3])
+@pytest.mark.parametrize("threads", [128, 256, 512])
+def test_parts_that_do_not_fit_shared_memory(tsx, blocks, threads):   # noqa: F811
+    A, b, c = lpgen.dense_lp(1900, 700, 3)
+    ref = _oracle_run(A, b, c, max_iters=40)
+    _assert_same(_gpu_run(tsx, A, b, c, path=1, max_iters=40, blocks=blocks, threads=threads), ref)
+
+
+@pytest.mark.parametrize("kw", [{"k_cyc": 3}, {"rule": 1}])
+def test_rules_with_pending_updates(tsx, kw):   # noqa: F811
+    A0, b0, c0 = lpgen.dense_lp(60, 45, 11)
+    A = np.vstack([A0, A0[:20], np.ones((3, 45))])
+    b = np.concatenate([b0, b0[:20], np.full(3, 50.0)])
+    _assert_same(_gpu_run(tsx, A, b, c0, path=1, **kw), _oracle_run(A, b, c0, **kw))
+
+
+# LPs whose scaled pivot row overflows after some pivots, with pivots after it
+# (a row of tiny entries and b = 0: the pivot element is ~1e-300); the last
+# pivot count stops right at the overflow
+@pytest.mark.parametrize("seed,first", [(10, 5), (147, 3), (183, 5), (336, 5)])
+def test_overflow_ends_a_round(tsx, seed, first):   # noqa: F811
+    rng = np.random.default_rng(seed)
+    A, b, c = lpgen.dense_lp(20, 15, seed)
+    A = A - 3.0
+    i = int(rng.integers(20))
+    b[i] = 0.0
+    A[i] *= 10.0 ** -rng.integers(290, 308)
+    A[i][rng.integers(15)] = 5
+    for k in (first, -1):
+        one = _gpu_run(tsx, A, b, c, path=1, eps_p=0.0, max_iters=k)
+        ref = _gpu_run(tsx, A, b, c, path=2, eps_p=0.0, max_iters=k)
+        assert not np.isfinite(ref[2]).all()
+        assert one[0] == ref[0] and one[1].iters == ref[1].iters
+        for x, y in zip((one[1].x, one[1].y, one[1].basis, *one[2:5]), (ref[1].x, ref[1].y, ref[1].basis, *ref[2:5])):
+            np.testing.assert_array_equal(x, y)
+        assert one[1].obj == ref[1].obj or (np.isnan(one[1].obj) and np.isnan(ref[1].obj))
