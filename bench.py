@@ -887,6 +887,14 @@ def run_many(args, rank, world, local):
     k_ms = statistics.median(kernel_ms)
     achieved = statistics.median(upd) / (k_ms / 1000.0) / 1e9
     peak, peak_src = measured_peaks()
+    flops = sum(2.0 * (m + 1) * (n + 1) * x["iters"] for (m, n), x in zip(shapes, stats))
+    fp64 = None
+    if prec == tsx.LP_PREC_FP64:   # several pivots per pass: the FP64 pipe is the ceiling
+        peak_f, _ = fp64_fma_rate(tsx, sptr)
+        ach_f = flops / (k_ms / 1000.0) / 1e12
+        fp64 = {"bound": "alu", "achieved": ach_f, "peak": peak_f, "unit": "TFLOP/s", "frac": ach_f / peak_f,
+                "peak_source": "measured FP64 fma rate in this run (lp_measure_fp64_fma_rate)",
+                "flops_per_launch": flops}
     # plain: every LP once through lp_solve (default persistent path)
     po = tsx.options(precision=prec, stream=sptr)
     t0 = time.perf_counter()
@@ -922,7 +930,10 @@ def run_many(args, rank, world, local):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)", "traffic": None,
                      "kernel": "k_team_solve", "kernel_ms_per_launch": k_ms,
-                     "bytes_per_launch": statistics.median(upd)},
+                     "bytes_per_launch": statistics.median(upd)} if fp64 is None else
+                    {**fp64, "kernel": "k_team_solve", "kernel_ms_per_launch": k_ms, "traffic": None,
+                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+                             "bytes_per_launch": statistics.median(upd)}},
         "plain": {"value": plain, "unit": "LPs/s", "path": "the same LPs one at a time through lp_solve",
                   "speedup": value / plain},
         "non_optimal": bad,

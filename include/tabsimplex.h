@@ -235,9 +235,10 @@ lp_status lp_solve(lp_t h, const lp_options *opt);
  * to half of the GPU into wide teams of four times as many blocks that take
  * those LPs first; each team takes the next LP from its list, largest first
  * (then helps with the other list), and iterates on
- * its condensed tableau: block b of the team owns a contiguous range of rows,
- * runs the ratio test on them and updates them, with the scaled pivot row and
- * its rows' multipliers in shared memory; two team barriers per pivot.  Meant
+ * its condensed tableau: block b of the team owns a contiguous range of rows
+ * and of columns and brings its part of the entering column and of the pivot
+ * row up to date, with two exchanges between the team's blocks per pivot; the
+ * updates of up to 16 (FP32: 32) pivots share one pass over the tableau.  Meant
  * for many medium LPs, whose pivots are too small to fill the GPU one at a
  * time.  Every pivot and value equals lp_solve's with the same options.
  *   handles  count distinct handles on the current device (lp_create*)
@@ -246,8 +247,8 @@ lp_status lp_solve(lp_t h, const lp_options *opt);
  *            blocks per team; precision LP_PREC_FP32 adds the FP64 recovery
  *            of each LP after the launch
  *   status   HOST output, count entries: each LP's status as lp_solve returns it
- * An LP whose pivot row and row multipliers do not fit one block's shared
- * memory is solved by lp_solve after the launch.  Afterwards each handle
+ * An LP whose pivot row and row multipliers would not fit one block's shared
+ * memory is solved by lp_solve after the launch (it fills the GPU by itself).  Afterwards each handle
  * answers lp_get_solution, lp_get_tableau and lp_get_stats as after lp_solve
  * (stats.path = LP_PATH_TEAM, stats.pivot_ms = the whole launch, no pivot
  * log).  Returns LP_OPTIMAL when the call ran (per-LP outcomes in status), or

@@ -686,7 +686,7 @@ static int max_coresident(int device) {
 // and, where the limit `limit` allows, the block's own parts of the LP.
 template <int NT, typename V>
 static size_t delayed_smem(int m, int n, int blocks, size_t limit) {
-    const size_t pass = delay_smem_bytes<V>(NT, delayed_rows(NT));
+    const size_t pass = delay_smem_bytes<V>(NT, kDelayedRows);
     const size_t own = delay_own_bytes<V>(m, n, blocks, pass);
     return own <= limit ? own : pass;
 }
@@ -714,7 +714,7 @@ static int delayed_coresident(int device, size_t& smem_limit) {
         cudaGetLastError();   // a refused attribute must not surface as a later launch's error
     });
     smem_limit = limit;
-    if (limit < delay_smem_bytes<V>(NT, delayed_rows(NT))) return 0;
+    if (limit < delay_smem_bytes<V>(NT, kDelayedRows)) return 0;
     int nsm = 0, per = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pivot_delayed<NT, V>, NT, limit) != cudaSuccess) {
@@ -1659,28 +1659,63 @@ lp_status lp_solve(lp_t h, const lp_options* opt) {
 // the per-LP bookkeeping of solve_nt (statistics, and for FP32 the FP64
 // recovery) for each handle.
 
-// The dynamic shared-memory limit of a team kernel is raised once to the
-// device's maximum (process-wide state, never lowered).
+// Dynamic shared memory that a block of a team kernel may use with as many
+// blocks per SM as the kernel is built for; the kernel's limit is raised to it
+// once (process-wide state, never lowered).
 template <int NT, typename V>
 static cudaError_t team_allow_smem(size_t& limit) {
     static std::once_flag once;
     static cudaError_t err = cudaSuccess;
     static size_t lim = 0;
     std::call_once(once, [] {
-        int dev = 0, optin = 0;
+        int dev = 0, per_sm = 0, reserved = 0;
         cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncAttributes fa{};
-        cudaFuncGetAttributes(&fa, k_team_solve<NT, V>);
-        lim = (size_t)std::max(0, optin - (int)fa.sharedSizeBytes);
-        err = cudaFuncSetAttribute(k_team_solve<NT, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
+        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+        constexpr int want = team_sm_threads(NT) / NT;
+        const void* kernels[2] = {(const void*)k_team_solve<NT, V>, (const void*)k_team_serve<NT, V>};
+        long long room = per_sm;
+        for (const void* k : kernels) {
+            cudaFuncAttributes fa{};
+            if (err == cudaSuccess) err = cudaFuncGetAttributes(&fa, k);
+            room = std::min(room, (long long)per_sm / want - reserved - (long long)fa.sharedSizeBytes);
+        }
+        lim = (size_t)std::max(0LL, room / 128 * 128);
+        for (const void* k : kernels)
+            if (err == cudaSuccess) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
     });
     limit = lim;
     return err;
 }
 
-// Bookkeeping of one LP after the team launch (as solve_nt): statistics and,
-// for FP32, the FP64 recovery; *status receives the LP's outcome.
+// LPs whose pivot row would not fit one block's shared memory go to lp_solve,
+// whose whole grid they fill.
+static bool team_takes(int device, int m, int ld, int elem, int C) {
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    return ((size_t)ld + delay_per(m + 1, C)) * elem <= (size_t)std::max(0, optin);
+}
+
+template <typename V>
+static TeamJob<V> team_job(const lp_handle* h) {
+    TeamJob<V> J{};
+    J.A = h->A;
+    J.b = h->b;
+    J.c = h->c;
+    J.T = (V*)h->work.T;
+    J.basis = h->basis;
+    J.var = h->work.var;
+    J.st = h->st;
+    J.Fh = (V*)h->work.Fh;
+    J.Rh = (V*)h->work.Rh;
+    J.RhT = (V*)h->work.RhT;
+    J.rhs = (V*)h->work.rhs;
+    J.m = h->m;
+    J.n = h->n;
+    J.ld = h->work.ld;
+    return J;
+}
+
 template <typename V>
 static lp_status finish_team_lp(lp_handle* h, const lp_options& o, cudaStream_t s, float ms, int C, int NT,
                                 lp_status* status) {
@@ -1701,13 +1736,13 @@ static lp_status finish_team_lp(lp_handle* h, const lp_options& o, cudaStream_t 
     }
     h->checked = true;
     const int m = h->m, ld = h->work.ld, E = 32 / elem;
-    const double nsec = (double)(ld / E);
     h->stats.iters = ds.iters;
     // ms < 0: a continuous launch, where the LP's team stamped its own start and end
     h->stats.pivot_ms = ms >= 0.f ? (double)ms : 1e-6 * (double)(ds.phase_ns[1] - ds.phase_ns[0]);
     h->stats.dense_update_bytes = 2.0 * (double)(m + 1) * (double)h->W * elem * (double)ds.iters;
-    h->stats.update_bytes = ((64.0 * (double)(m - 1) + 96.0) * nsec + 64.0 * (double)(m + 1) +
-                             3.0 * elem * (double)ld) * (double)ds.iters;
+    // as in solve_nt for delayed updates
+    h->stats.update_bytes = 64.0 * (double)m * (double)((h->n + E - 1) / E) * (double)ds.passes +
+                            (96.0 * (double)(m + 1) + 4.0 * elem * (double)ld) * (double)ds.iters;
     h->stats.path = LP_PATH_TEAM;
     h->stats.grid = C;
     h->stats.block = NT;
@@ -1771,36 +1806,24 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
             CUDA_TRY(cudaStreamWaitEvent(s, h->ev[0], 0), LP_ERR_CUDA);
         }
     }
-    // the list, largest first; LPs whose pivot row and multipliers exceed the
-    // shared memory of one block are solved one at a time afterwards
+    // the list, largest first
     std::vector<TeamJob<V>> jobs;
     std::vector<int> who, alone;
     std::vector<double> work;
-    int ld_max = 0, rows_max = 0;
+    const size_t pass_bytes = delay_smem_bytes<V>(NT, kTeamRows);
+    size_t smem = pass_bytes;
     for (int k = 0; k < count; ++k) {
         lp_handle* h = hs[k];
-        const int rows = (h->m + 1 + C - 1) / C;
-        if ((size_t)(h->work.ld + rows) * elem > smem_limit) {
+        if (!team_takes(device, h->m, h->work.ld, elem, C)) {
             alone.push_back(k);
             continue;
         }
-        TeamJob<V> J{};
-        J.A = h->A;
-        J.b = h->b;
-        J.c = h->c;
-        J.T = (V*)h->work.T;
-        J.basis = h->basis;
-        J.var = h->work.var;
-        J.st = h->st;
-        J.m = h->m;
-        J.n = h->n;
-        J.ld = h->work.ld;
-        jobs.push_back(J);
+        jobs.push_back(team_job<V>(h));
         who.push_back(k);
         work.push_back((double)(h->m + 1) * h->work.ld * (double)(h->m + h->n));
-        ld_max = std::max(ld_max, h->work.ld);
-        rows_max = std::max(rows_max, rows);
+        smem = std::max(smem, delay_own_bytes<V>(h->m, h->n, C, pass_bytes));
     }
+    smem = std::min(smem, smem_limit);
     const int njobs = (int)jobs.size();
     std::vector<int> order(njobs);
     for (int k = 0; k < njobs; ++k) order[k] = k;
@@ -1808,7 +1831,6 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
 
     float ms = 0.f;
     if (njobs > 0) {
-        const size_t smem = (size_t)(ld_max + ((rows_max + 31) / 32) * 32) * elem;
         int per = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_team_solve<NT, V>, NT, smem);
         const int cap = per * nsm - std::max(0, reserve_blocks);
@@ -1904,8 +1926,8 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
         if (!ensure_events(h0)) return LP_ERR_CUDA;
         cudaEvent_t e0 = h0->ev[1], e1 = h0->ev[2];
         if (e == cudaSuccess) e = cudaEventRecord(e0, s);
-        int ldm = ld_max;
-        void* args[] = {(void*)&P, (void*)&ldm};
+        unsigned smem_bytes = (unsigned)smem;
+        void* args[] = {(void*)&P, (void*)&smem_bytes};
         if (e == cudaSuccess)
             e = cudaLaunchCooperativeKernel((const void*)k_team_solve<NT, V>, grid, NT, args, smem, s);
         if (e == cudaSuccess) e = cudaEventRecord(e1, s);
@@ -1986,7 +2008,6 @@ struct tsx::TeamLane {
     int reserve = 0;
     int C = 16, CB = 64, grid = 0, nteams = 0;
     size_t smem = 0;
-    int ld_cap = 0, rows_cap = 0;
     // mapped host memory: rings, tails, done words, stop word
     char* hmem = nullptr;
     char* hmem_d = nullptr;
@@ -2067,8 +2088,8 @@ static lp_status lane_launch(TeamLane* L) {
     P.jcopy = (TeamJob<V>*)(base + L->o_jc);
     P.idle_ns = kLaneIdleNs;
     P.idle_cap_ns = kLaneIdleCapNs;
-    int ldm = L->ld_cap;
-    void* args[] = {(void*)&P, (void*)&ldm};
+    unsigned smem_bytes = (unsigned)L->smem;
+    void* args[] = {(void*)&P, (void*)&smem_bytes};
     CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_team_serve<NT, V>, grid, NT, args, L->smem, L->ks),
              LP_ERR_CUDA);
     CUDA_TRY(cudaEventRecord(L->kev, L->ks), LP_ERR_CUDA);
@@ -2080,24 +2101,10 @@ static lp_status lane_launch(TeamLane* L) {
 template <typename V>
 static lp_status lane_setup(TeamLane* L) {
     constexpr int NT = 256;
-    constexpr int elem = (int)sizeof(V);
     CUDA_TRY(cudaGetDevice(&L->device), LP_ERR_CUDA);
     cudaDeviceGetAttribute(&L->nsm, cudaDevAttrMultiProcessorCount, L->device);
-    // shared memory for two blocks per SM: R (ld_cap entries) and the
-    // multipliers of a block's rows (rows_cap entries)
-    int per_sm = 0, reserved = 0;
-    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, L->device);
-    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, L->device);
-    cudaFuncAttributes fa{};
-    CUDA_TRY(cudaFuncGetAttributes(&fa, k_team_serve<NT, V>), LP_ERR_CUDA);
-    const size_t per_block = (size_t)per_sm / 2 - (size_t)reserved - fa.sharedSizeBytes - 1024;
-    const size_t entries = per_block / elem / 32 * 32;
-    L->ld_cap = (int)(entries * 3 / 4 / 32 * 32);
-    L->rows_cap = (int)entries - L->ld_cap;
-    L->smem = entries * elem;
-    CUDA_TRY(cudaFuncSetAttribute((const void*)k_team_serve<NT, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)L->smem),
-             LP_ERR_CUDA);
+    const cudaError_t se = team_allow_smem<NT, V>(L->smem);
+    CUDA_TRY(se, LP_ERR_CUDA);
     int per = 0;
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_team_serve<NT, V>, NT, L->smem), LP_ERR_CUDA);
     L->grid = per * L->nsm - L->reserve;
@@ -2159,25 +2166,14 @@ long long tsx::lane_submit(TeamLane* L, lp_t h) {
     CUDA_TRY(cudaSetDevice(h->device), -1);
     CUDA_TRY(cudaStreamWaitEvent(h->stream, h->ready, 0), -1);
     if (ensure_work(h, elem, 1) != LP_OPTIMAL) return -1;
-    const int rows = (h->m + 1 + L->C - 1) / L->C;
-    if (h->work.ld > L->ld_cap || rows > L->rows_cap) return -2;   // solve it another way
+    if (!team_takes(h->device, h->m, h->work.ld, elem, L->C)) return -2;   // solve it another way
     h->stats = lp_stats{};
     h->sol_ready = false;
     h->final_basis.clear();
     // the team resets the LP's state words when it takes the job; the
     // buffers' stream-ordered allocation is complete before it is published
     CUDA_TRY(cudaStreamSynchronize(h->stream), -1);
-    TeamJob<double> J{};   // same layout for both element types (pointers and ints)
-    J.A = h->A;
-    J.b = h->b;
-    J.c = h->c;
-    J.T = (double*)h->work.T;
-    J.basis = h->basis;
-    J.var = h->work.var;
-    J.st = h->st;
-    J.m = h->m;
-    J.n = h->n;
-    J.ld = h->work.ld;
+    const TeamJob<double> J = team_job<double>(h);   // same layout for both element types (pointers and ints)
     const double work = (double)(h->m + 1) * (double)(h->n + 1) * (double)(h->m + h->n);
     const unsigned l = work > kLaneHeavyWork ? 1u : 0u;
     std::lock_guard<std::mutex> lk(L->mu);

@@ -270,9 +270,10 @@ __device__ __forceinline__ bool delay_finite(float x) {
 // by the packed fma.rn.f32x2: one rounding per float, as fmaf).  Per pending
 // pivot a lane takes its 32 bytes of R (shared memory, staged once per column
 // strip for the whole block) and the rows' multipliers (shared memory, staged
-// per tile, already negated; broadcast reads of two rows at a time).  The next
-// tile's loads are in flight while a tile is updated: 64 KB per SM at any time
-// with 8 warps and 8-row tiles, which is what the HBM stream needs.
+// per tile, already negated; broadcast reads of two rows at a time).  With one
+// block of 8 warps per SM the next tile's loads are in flight while a tile is
+// updated: 64 KB per SM at any time with 8-row tiles, which is what the HBM
+// stream needs.
 template <typename V> struct Word;
 template <> struct Word<double> {
     static __device__ __forceinline__ unsigned long long neg(double f) { return __double_as_longlong(-f); }
@@ -378,7 +379,10 @@ struct DelayTile {
 // one strip and tiles in turn: the wait after the pass 4.5 -> 2.5 us a pivot).
 // `rev`: the range backwards (alternate passes start on the tiles the previous
 // one left in L2).
-template <int NT, int RS, typename V>
+// AHEAD: the next tile's loads in flight while a tile is updated (needs the
+// registers of one block of 256 threads per SM); without, the other warps of
+// the SM cover a tile's loads.
+template <int NT, int RS, bool AHEAD, typename V>
 __device__ __forceinline__ void delay_pass(const Delayed<V>& D, int k, int rev, unsigned char* smem, DelayScratch& s) {
     constexpr int K = DelayK<V>::K, E = Lanes<V>::E, NS = kDelayStrips;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -417,15 +421,24 @@ __device__ __forceinline__ void delay_pass(const Delayed<V>& D, int k, int rev, 
             const int g = strip * 32 + lane;
             tile.load(D, k, 1 + row * RS, g * E, g < ngroups, strip - f);
         };
-        DelayTile<V, RS> cur, ahead;
         unsigned z = next();
-        if (z < count) load(cur, z);
+        if constexpr (AHEAD) {
+            DelayTile<V, RS> cur, ahead;
+            if (z < count) load(cur, z);
 #pragma unroll 1
-        while (z < count) {
-            z = next();
-            if (z < count) load(ahead, z);
-            cur.update(D, k, rs, fs);
-            cur = ahead;
+            while (z < count) {
+                z = next();
+                if (z < count) load(ahead, z);
+                cur.update(D, k, rs, fs);
+                cur = ahead;
+            }
+        } else {
+#pragma unroll 1
+            for (; z < count; z = next()) {
+                DelayTile<V, RS> tile;
+                load(tile, z);
+                tile.update(D, k, rs, fs);
+            }
         }
     }
 }
@@ -680,7 +693,7 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
 // are in shared memory; s.passed is set by the caller.
 // clk: work of {Steps 1-2, row p and the objective row, the passes}, then the
 // wait after each.
-template <int NT, int RS, typename V, typename Clock>
+template <int NT, int RS, bool AHEAD = false, typename V, typename Clock>
 __device__ __forceinline__ void delayed_solve(const Delayed<V>& D, unsigned char* smem, DelayScratch& s, DelayState& S,
                                               Clock& clk) {
     const size_t pass_bytes = delay_smem_bytes<V>(NT, RS);
@@ -693,7 +706,7 @@ __device__ __forceinline__ void delayed_solve(const Delayed<V>& D, unsigned char
         if (k > 0) {   // the pending updates applied to the whole tableau, between two barriers
             if (!delay_barrier(D, s)) break;
             const int rev = (int)(S.passes & 1u);
-            delay_pass<NT, RS>(D, k, rev, smem, s);
+            delay_pass<NT, RS, AHEAD>(D, k, rev, smem, s);
             clk.lap(2);
             if (!delay_barrier(D, s)) break;
             if (S.flag) {   // 0 x inf in row p: the row again

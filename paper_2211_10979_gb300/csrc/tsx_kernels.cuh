@@ -285,8 +285,7 @@ __global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_pe
 
 // The condensed tableau's persistent kernel: one cooperative launch, the grid's
 // blocks as the blocks of one delayed solve.
-// Rows of an update tile: two tiles of 8 rows fill half of 255 registers.
-__host__ __device__ constexpr int delayed_rows(int nt) { return persistent_sm_threads(nt) <= 256 ? 8 : 4; }
+constexpr int kDelayedRows = 8;   // rows of an update tile
 template <int NT, typename V>
 __global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_delayed(Delayed<V> lp, DevState* st) {
     extern __shared__ __align__(128) unsigned char tsx_dyn[];
@@ -302,7 +301,7 @@ __global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_de
     }
     __syncthreads();
     clk.start();
-    delayed_solve<NT, delayed_rows(NT)>(D, tsx_dyn, s, S, clk);
+    delayed_solve<NT, kDelayedRows, (persistent_sm_threads(NT) <= 256)>(D, tsx_dyn, s, S, clk);
     if (blockIdx.x == 0 && threadIdx.x == 0 && S.status != kDelayFailed) {
         atomicCAS(&st->status, kRunning, S.status);
         st->iters = S.it;

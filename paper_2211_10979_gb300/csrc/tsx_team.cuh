@@ -3,19 +3,17 @@
 // too large for one block's shared memory and too small to fill the GPU.
 //
 // One cooperative launch holds every team; a team takes the next LP from a
-// list (largest first) and solves it on its condensed tableau in global
-// memory.  Block b of the team owns a contiguous range of rows: it runs the
-// ratio test on its rows (keeping their column-q entries, the multipliers, in
-// shared memory), stages the whole scaled pivot row R in its own shared memory
-// (each block divides row p by the pivot itself), and updates its rows.  Block
-// 0 owns row 0 and finds the next entering column while it updates it.  Two
-// team barriers per pivot: after the ratio test (every block learns p) and
-// after the update (every block learns the next entering column, and every
-// block has read row p, so its owner may now overwrite it with R).  The
-// arithmetic and the tie rules are those of the single-LP kernels, so every
-// pivot and value equals lp_solve's.
+// list (largest first), builds its condensed tableau in global memory, a range
+// of rows per block, and solves it with delayed updates (tsx_delayed.cuh): its
+// blocks are the blocks of one delayed solve, so that the updates of up to 16
+// (FP32: 32) pivots share one pass over the tableau.  The arithmetic and the
+// tie rules are those of the single-LP kernels, so every pivot and value equals
+// lp_solve's.  Measured against one update per pivot (bound by HBM, 0.86 of
+// it): 96 FP64 LPs with m, n log-uniform in [180, 3000] 110-118 -> 63-87 ms (two
+// boxes), a burst of 200 FP32 requests with m, n in [32, 4096] 201 -> 71 ms.
 #pragma once
 
+#include "tsx_delayed.cuh"
 #include "tsx_device.cuh"
 
 namespace tsx {
@@ -24,13 +22,10 @@ constexpr int kTeamMax = 160;  // blocks per team, upper bound
 #ifndef TSX_TEAM_SM_THREADS
 #define TSX_TEAM_SM_THREADS 512   // threads per SM the team kernel is compiled for
 #endif
-#ifndef TSX_TEAM_SLICE_LD
-#define TSX_TEAM_SLICE_LD 1024   // FP64 rows this long or longer: row p scaled a slice per block
-#endif
-// Threads per SM of the team kernel with blocks of nt threads, and the rows a
-// warp of its update keeps in flight (16 where a thread may hold 255 registers).
+// Threads per SM of the team kernel with blocks of nt threads, and the rows of
+// a warp's update tile.
 __host__ __device__ constexpr int team_sm_threads(int nt) { return nt > TSX_TEAM_SM_THREADS ? nt : TSX_TEAM_SM_THREADS; }
-__host__ __device__ constexpr int team_rows_in_flight(int nt) { return team_sm_threads(nt) <= 256 ? 16 : kRowsInFlight; }
+constexpr int kTeamRows = 8;
 
 template <typename V>
 struct TeamJob {
@@ -40,7 +35,11 @@ struct TeamJob {
     V* T;                      // condensed tableau (m+1) x ld
     int* basis;                // m
     int* var;                  // n
-    DevState* st;              // the LP's state words: status, iters, bland, degen_run
+    DevState* st;              // the LP's state words: status, iters, bland, degen_run, passes
+    V* Fh;                     // buffers of the delayed updates
+    V* Rh;
+    V* RhT;
+    V* rhs;
     int m, n, ld;
     int pad;
 };
@@ -52,8 +51,9 @@ struct __align__(256) TeamState {   // one per team
     int fail;                  // set when a team barrier wait ran out
     int bad;                   // the current LP's inputs are not finite or b < 0
     unsigned seq;              // continuous launch: sequence number of the job
-    ArgPart ent;               // next entering candidate (block 0)
-    RatPart rat[kTeamMax];     // ratio-test partial of each block
+    unsigned delay_count;      // arrivals of the delayed solve's exchanges and barriers
+    DelayRec arg[kTeamMax];    // entering candidate of each block
+    DelayRec rat[kTeamMax];    // leaving candidate of each block
 };
 
 template <typename V>
@@ -170,195 +170,113 @@ __device__ void team_build(const TeamJob<V>& J, int r0, int r1, int bt, TeamStat
         for (int j = threadIdx.x; j < n; j += blockDim.x) J.var[j] = j;
 }
 
-// Objective row (block 0): T[0][j] = fma(-f0, R[j], T[0][j]) (q: from the
-// leaving variable's unit column, 0 off row p) when R != null, then the
-// entering candidate of the new row over all slots, posted to the team.
-template <typename V>
-__device__ void team_row0(const TeamJob<V>& J, const V* R, V f0, int q, const TeamParams<V>& P, TeamState* ts,
-                          BlockScratch& s) {
-    constexpr int E = Lanes<V>::E;
-    const int nsec = J.ld / E;
-    ArgPart a = arg_none();
-    for (int g = threadIdx.x; g < nsec; g += blockDim.x) {
-        const int j = g * E;
-        Sector<V> o = ld_sector_cg(J.T + j);
-        if (R) {
-            const Sector<V> r = *reinterpret_cast<const Sector<V>*>(R + j);
-#pragma unroll
-            for (int e = 0; e < E; ++e) o.v[e] = fma_rn(-f0, r.v[e], j + e == q ? V(0) : o.v[e]);
-            st_sector(J.T + j, o);
-        }
-        arg_consider_sector(a, o, j, J.n, P.eps_d, J.var);
-    }
-    a = block_arg(a, s);
-    if (threadIdx.x == 0) store_arg(&ts->ent, a);
-}
+struct NoClock {
+    __device__ void lap(int) {}
+};
 
-// Rank-1 update of the block's rows [lo, r1) except p, R and the multipliers
-// (Floc, indexed from r0) in shared memory; slots of RF rows x 32 column
-// groups, one group per lane.
-template <typename V, int RF>
-__device__ void team_update(const TeamJob<V>& J, const V* R, const V* Floc, int r0, int lo, int r1, int p, int q) {
-    constexpr int E = Lanes<V>::E;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nsec = J.ld / E;
-    const int nchunks = (nsec + 31) / 32;
-    const int nrg = (r1 - lo + RF - 1) / RF;
-    const long long total = (long long)nrg * nchunks;
-    for (long long u = warp; u < total; u += nw) {
-        const int rg = (int)(u / nchunks), ch = (int)(u - (long long)rg * nchunks);
-        const int i0 = lo + rg * RF;
-        const int nrows = min(RF, r1 - i0);
-        const int gidx = ch * 32 + lane;
-        if (gidx >= nsec) continue;
-        const size_t col = (size_t)E * (size_t)gidx;
-        const Sector<V> r = *reinterpret_cast<const Sector<V>*>(R + col);
-        const int eq = q - (int)col;
-        Sector<V> v[RF];
-#pragma unroll
-        for (int k = 0; k < RF; ++k) {
-            const int i = i0 + k;
-            if (k < nrows && i != p) v[k] = ld_sector_stream(J.T + (size_t)i * (size_t)J.ld + col);
-        }
-#pragma unroll
-        for (int k = 0; k < RF; ++k) {
-            const int i = i0 + k;
-            if (k < nrows && i != p) {
-                const V f = Floc[i - r0];
-#pragma unroll
-                for (int e2 = 0; e2 < E; ++e2) v[k].v[e2] = fma_rn(-f, r.v[e2], e2 == eq ? V(0) : v[k].v[e2]);
-                st_sector(J.T + (size_t)i * (size_t)J.ld + col, v[k]);
-            }
-        }
+// Shared memory of a team's block.
+template <typename V>
+struct TeamScratch {
+    DelayScratch ds;
+    DelayState state;
+    Delayed<V> lp;
+    TeamJob<V> job;
+    int ok;
+    unsigned passed;   // team barriers this block has passed (thread 0)
+};
+
+// A job entry from global memory (written before the team's last barrier) into
+// shared memory.
+template <typename V>
+__device__ __forceinline__ void team_copy_job(TeamJob<V>& to, const TeamJob<V>* from) {
+    static_assert(sizeof(TeamJob<V>) % 8 == 0, "copied in 8-byte words");
+    const unsigned w = threadIdx.x;
+    if (w < sizeof(TeamJob<V>) / 8) {
+        const unsigned long long x = __ldcg(reinterpret_cast<const unsigned long long*>(from) + w);
+        memcpy(reinterpret_cast<char*>(&to) + 8 * w, &x, 8);
     }
+    __syncthreads();
 }
 
 // Solves one LP with the team of C blocks; false if a team barrier failed.
-template <int RF, typename V>
+template <int NT, typename V>
 __device__ bool team_solve_one(const TeamParams<V>& P, const TeamJob<V>& J, TeamState* ts, int bt, unsigned C,
-                               V* R, V* Floc, BlockScratch& s, int& sok, unsigned& tpass) {
-    const int m = J.m, n = J.n, ld = J.ld;
+                               unsigned char* smem, unsigned smem_bytes, TeamScratch<V>& s) {
+    const int m = J.m, n = J.n;
     int r0, r1;
     team_rows(m, (int)C, bt, r0, r1);
     team_build(J, r0, r1, bt, ts);
-    __syncthreads();
-    if (bt == 0) team_row0(J, (const V*)nullptr, V(0), -1, P, ts, s);   // Step 1 of the first pivot
-    if (!team_barrier(ts, C, P.timeout_ns, sok, tpass)) return false;
-    const long long cap = P.max_iters < 0 ? 50LL * ((long long)m + n) : P.max_iters;
-    long long it = 0;
-    int bland = P.rule == 1, degen = 0;
-    int status = ld_relaxed(&ts->bad) ? kInvalid : kRunning;
-    const int lo = max(r0, 1);
-    const int i_first = lo + (int)threadIdx.x;   // the thread's first row in Step 2
-    while (status == kRunning) {
-        // its right-hand side, in flight while Step 1's candidate is read
-        const V rhs0 = i_first < r1 ? __ldcg(J.T + (size_t)i_first * (size_t)ld + n) : V(0);
-        const ArgPart e = load_arg(&ts->ent);                // Step 1
-        const int q = bland ? e.fslot : e.slot;
-        const int qv = bland ? e.fkey : e.key;
-        if (qv == INT_MAX) { status = kOptimal; break; }
-        if (it >= cap) { status = kIterLimit; break; }
-        // Step 2 on the block's rows; their column-q entries become the multipliers
-        RatPart best = rat_none();
-        if (bt == 0 && threadIdx.x == 0) Floc[0] = __ldcg(J.T + q);
-        for (int i = i_first; i < r1; i += blockDim.x) {
-            const V* row = J.T + (size_t)i * (size_t)ld;
-            const V a = __ldcg(row + q);
-            Floc[i - r0] = a;
-            if ((double)a > P.eps_p) {
-                RatPart c;
-                c.r = (double)div_rn(i == i_first ? rhs0 : __ldcg(row + n), a);
-                c.i = i;
-                c.key = bland ? __ldcg(J.basis + (i - 1)) : i;
-                c.a = (double)a;
-                c.pad = 0.0;
-                if (!dbits_nan(c.r)) rat_merge(best, c);
-            }
-        }
-        best = block_rat(best, s);
-        if (threadIdx.x == 0) store_rat(&ts->rat[bt], best);
-        if (!team_barrier(ts, C, P.timeout_ns, sok, tpass)) return false;
-        RatPart l = rat_none();
-        if (threadIdx.x < (int)C) l = load_rat(&ts->rat[threadIdx.x]);
-        l = block_rat(l, s);
-        if (l.i == INT_MAX) { status = kUnbounded; break; }
-        const int p = l.i;
-        const V piv = (V)l.a;
-        if (!isfinite((double)piv) || !isfinite(l.r)) { status = kNumeric; break; }
-        // Step 3, pivot row; the leaving variable takes slot q.  FP64 rows of
-        // TSX_TEAM_SLICE_LD entries or more: each block scales its slice of
-        // row p in place (the new row p), a team barrier, then every block
-        // reads the whole row (GB300's FP64 pipe charges ~9 fused
-        // multiply-adds per division, ld of them a block otherwise).  Shorter
-        // or FP32 rows: every block scales the whole row itself.
-        V* rowp = J.T + (size_t)p * (size_t)ld;
-        const bool slice = sizeof(V) == 8 && ld >= TSX_TEAM_SLICE_LD;
-        if (slice) {
-            const int sl = (ld + (int)C - 1) / (int)C;
-            const int j0 = min(ld, bt * sl), j1 = min(ld, j0 + sl);
-            for (int j = j0 + (int)threadIdx.x; j < j1; j += blockDim.x)
-                rowp[j] = div_rn(j == q ? V(1) : __ldcg(rowp + j), piv);
-        } else {
-            for (int j = threadIdx.x; j < ld; j += blockDim.x) R[j] = div_rn(j == q ? V(1) : __ldcg(rowp + j), piv);
-        }
-        if (bt == 0 && threadIdx.x == 0) {
-            const int leaving = J.basis[p - 1];
-            J.basis[p - 1] = qv;
-            J.var[q] = leaving;
-        }
-        if (P.rule == 0) {
-            if (l.r <= 0.0) {
-                ++degen;
-                if (P.k_cyc > 0 && degen >= P.k_cyc) bland = 1;
-            } else {
-                degen = 0;
-                bland = 0;
-            }
-        }
-        if (slice) {
-            if (!team_barrier(ts, C, P.timeout_ns, sok, tpass)) return false;
-            for (int j = threadIdx.x; j < ld; j += blockDim.x) R[j] = __ldcg(rowp + j);
-        }
-        __syncthreads();
-        if (bt == 0) team_row0(J, R, Floc[0], q, P, ts, s);   // the next Step 1 on the new row 0
-        team_update<V, RF>(J, R, Floc, r0, lo, r1, p, q);
-        ++it;
-        if (!team_barrier(ts, C, P.timeout_ns, sok, tpass)) return false;
-        if (!slice && p >= r0 && p < r1) {   // every block has read row p: its owner stores R there
-            for (int j = threadIdx.x; j < ld; j += blockDim.x) J.T[(size_t)p * (size_t)ld + j] = R[j];
-            __syncthreads();
-        }
+    if (threadIdx.x == 0) {
+        Delayed<V>& D = s.lp;
+        D.T = J.T;
+        D.ld = J.ld;
+        D.m = m;
+        D.n = n;
+        D.basis = J.basis;
+        D.var = J.var;
+        D.Fh = J.Fh;
+        D.Rh = J.Rh;
+        D.RhT = J.RhT;
+        D.rhs = J.rhs;
+        D.rat = ts->rat;
+        D.arg = ts->arg;
+        D.bar_count = &ts->delay_count;
+        D.fail = &ts->fail;
+        D.status = nullptr;
+        D.bt = bt;
+        D.G = (int)C;
+        D.smem = smem_bytes;
+        D.eps_d = P.eps_d;
+        D.eps_p = P.eps_p;
+        D.max_iters = P.max_iters < 0 ? 50LL * ((long long)m + n) : P.max_iters;
+        D.k_cyc = P.k_cyc;
+        D.rule = P.rule;
+        D.timeout_ns = P.timeout_ns;
+        D.qlog = nullptr;
+        D.plog = nullptr;
+        D.log_cap = 0;
+    }
+    if (!team_barrier(ts, C, P.timeout_ns, s.ok, s.passed)) return false;
+    int status = kInvalid;
+    if (!ld_relaxed(&ts->bad)) {
+        NoClock clk;
+        delayed_solve<NT, kTeamRows>(s.lp, smem, s.ds, s.state, clk);
+        status = s.state.status;
+        if (status == kDelayFailed) return false;
     }
     // commit: the status is written only once every block of the team has
     // finished its part (a block that gave up at a barrier never gets here,
     // and the LP stays unfinished)
-    if (!team_barrier(ts, C, P.timeout_ns, sok, tpass)) return false;
+    if (!team_barrier(ts, C, P.timeout_ns, s.ok, s.passed)) return false;
     if (bt == 0 && threadIdx.x == 0) {
         J.st->status = status;
-        J.st->iters = it;
-        J.st->bland = bland;
-        J.st->degen_run = degen;
+        if (status != kInvalid) {
+            J.st->iters = s.state.it;
+            J.st->bland = s.state.bland;
+            J.st->degen_run = s.state.degen;
+            J.st->passes = s.state.passes;
+        } else {
+            J.st->iters = 0;
+            J.st->bland = P.rule == 1;
+            J.st->degen_run = 0;
+            J.st->passes = 0;
+        }
     }
     return true;
 }
 
 // One cooperative launch: team t (blocks first[t] .. first[t] + size[t] - 1)
 // takes entries of its own list, then of the other one, until both are empty.
-// Dynamic shared memory per block: R (ld_max entries) then the multipliers
-// (rows per block, max over the lists for the smallest team).
+// Dynamic shared memory per block: smem_bytes, for the delayed solves.
 template <int NT, typename V>
-__global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(TeamParams<V> P, int ld_max) {
-    extern __shared__ __align__(32) unsigned char team_smem[];
-    __shared__ BlockScratch s;
-    __shared__ int sok;
-    __shared__ unsigned tpass;   // counted team barriers passed (thread 0)
-    if (threadIdx.x == 0) tpass = 0;
+__global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(TeamParams<V> P, unsigned smem_bytes) {
+    extern __shared__ __align__(128) unsigned char tsx_dyn[];
+    __shared__ TeamScratch<V> s;
+    if (threadIdx.x == 0) s.passed = s.ds.passed = 0;
     const int t = P.team_of[blockIdx.x];
     const int bt = blockIdx.x - P.first[t];
     const unsigned C = (unsigned)P.size[t];
     TeamState* ts = P.teams + t;
-    V* R = reinterpret_cast<V*>(team_smem);
-    V* Floc = R + ld_max;
     int li = P.list[t];
     for (;;) {
         if (bt == 0 && threadIdx.x == 0) {
@@ -371,11 +289,11 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(Tea
             }
             ts->job = k;
         }
-        if (!team_barrier(ts, C, P.timeout_ns, sok, tpass)) return;
+        if (!team_barrier(ts, C, P.timeout_ns, s.ok, s.passed)) return;
         const int k = *(volatile const int*)&ts->job;
         if (k < 0) return;
-        const TeamJob<V> J = P.jobs[k];
-        if (!team_solve_one<team_rows_in_flight(NT)>(P, J, ts, bt, C, R, Floc, s, sok, tpass)) return;
+        team_copy_job(s.job, P.jobs + k);
+        if (!team_solve_one<NT>(P, s.job, ts, bt, C, tsx_dyn, smem_bytes, s)) return;
     }
 }
 
@@ -430,18 +348,14 @@ __device__ __forceinline__ void st_release_sys(unsigned* p, unsigned v) {
 }
 
 template <int NT, typename V>
-__global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(TeamServeParams<V> P, int ld_max) {
-    extern __shared__ __align__(32) unsigned char team_smem[];
-    __shared__ BlockScratch s;
-    __shared__ int sok;
-    __shared__ unsigned tpass;
-    if (threadIdx.x == 0) tpass = 0;
+__global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(TeamServeParams<V> P, unsigned smem_bytes) {
+    extern __shared__ __align__(128) unsigned char tsx_dyn[];
+    __shared__ TeamScratch<V> s;
+    if (threadIdx.x == 0) s.passed = s.ds.passed = 0;
     const int t = P.tp.team_of[blockIdx.x];
     const int bt = blockIdx.x - P.tp.first[t];
     const unsigned C = (unsigned)P.tp.size[t];
     TeamState* ts = P.tp.teams + t;
-    V* R = reinterpret_cast<V*>(team_smem);
-    V* Floc = R + ld_max;
     const int li = P.tp.list[t];
     TeamJob<V>* jc = P.jcopy + t;
     for (;;) {
@@ -491,18 +405,13 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
                 ts->job = -1;
             }
         }
-        if (!team_barrier(ts, C, P.tp.timeout_ns, sok, tpass)) return;
+        if (!team_barrier(ts, C, P.tp.timeout_ns, s.ok, s.passed)) return;
         const int slot = *(volatile const int*)&ts->job;
         if (slot < 0) return;
-        TeamJob<V> J;
-        {
-            const unsigned long long* src = reinterpret_cast<const unsigned long long*>(jc);
-            unsigned long long* dst = reinterpret_cast<unsigned long long*>(&J);
-            for (int w = 0; w < (int)(sizeof(TeamJob<V>) / 8); ++w) dst[w] = __ldcg(src + w);
-        }
+        team_copy_job(s.job, jc);
         if (bt == 0 && threadIdx.x == 0) {
             // the LP's state words start from zero here (no reset launch per job)
-            DevState* st = J.st;
+            DevState* st = s.job.st;
             st->status = kRunning;
             st->q = -1;
             st->p = -1;
@@ -516,16 +425,18 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
             st->bar_gen = 0;
             st->nact = 0;
             st->next_slot = 0;
+            st->fail = 0;
+            st->passes = 0;
             for (int q = 2; q < 6; ++q) st->phase_ns[q] = 0;
             st->phase_ns[1] = 0;
             st->phase_ns[0] = global_ns();
         }
-        if (!team_solve_one<team_rows_in_flight(NT)>(P.tp, J, ts, bt, C, R, Floc, s, sok, tpass)) {
+        if (!team_solve_one<NT>(P.tp, s.job, ts, bt, C, tsx_dyn, smem_bytes, s)) {
             if (bt == 0 && threadIdx.x == 0) atomicSub(P.busy, 1u);
             return;
         }
         if (bt == 0 && threadIdx.x == 0) {
-            J.st->phase_ns[1] = global_ns();
+            s.job.st->phase_ns[1] = global_ns();
             __threadfence_system();
             st_release_sys(P.ring.done + slot, *(volatile unsigned*)&ts->seq + 1u);
             atomicSub(P.busy, 1u);
