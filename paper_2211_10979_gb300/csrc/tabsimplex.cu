@@ -725,7 +725,7 @@ static int delayed_coresident(int device, size_t& smem_limit) {
 }
 
 template <typename V>
-static Delayed<V> delayed_params(lp_handle* h, const lp_options& o, double eps_d, double eps_p) {
+static Delayed<V> delayed_params(lp_handle* h, const lp_options& o) {
     Delayed<V> D{};
     D.T = (V*)h->work.T;
     D.ld = h->work.ld;
@@ -742,8 +742,6 @@ static Delayed<V> delayed_params(lp_handle* h, const lp_options& o, double eps_d
     D.bar_count = &h->st->bar_count;
     D.fail = &h->st->fail;
     D.status = &h->st->status;
-    D.eps_d = eps_d;
-    D.eps_p = eps_p;
     D.max_iters = o.max_iters < 0 ? 50LL * ((long long)h->m + h->n) : o.max_iters;
     D.k_cyc = o.k_cyc;
     D.rule = o.rule;
@@ -1190,13 +1188,13 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     if (path == LP_PATH_PERSISTENT) {
         cudaError_t e = cudaSuccess;
         if (dgrid) {
-            Delayed<V> D = delayed_params<V>(h, o, eps_d, eps_p);
+            Delayed<V> D = delayed_params<V>(h, o);
             D.smem = (unsigned)dsmem;
             D.qlog = P.qlog;
             D.plog = P.plog;
             D.log_cap = P.log_cap;
             DevState* st = h->st;
-            void* args[] = {(void*)&D, (void*)&st};
+            void* args[] = {(void*)&D, (void*)&eps_d, (void*)&eps_p, (void*)&st};
             grid_run = dgrid;
             e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
         } else {

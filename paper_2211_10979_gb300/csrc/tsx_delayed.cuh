@@ -26,10 +26,10 @@
 // pivot (8192^2 FP64: 151 of 166 us a pivot; 12288^2 FP32: 172 of 178 us).
 // Delayed, that traffic is divided by K and the pass is bound by its fused
 // multiply-adds (FP64 pipe: 626 G fma/s), plus a latency chain per pivot of
-// two exchanges between the blocks (8-9 us).  Measured, undelayed -> delayed,
-// us a pivot: FP64 1024^2 15.3 -> 10.2, 4096^2 51 -> 36.6 (pass 26.8, its fmas
-// alone 26.8), 8192^2 166 -> 118.5 (pass 108.7, its fmas 107.2); FP32 4096^2
-// 33 -> 9.1, 12288^2 178 -> 18.4 (pass 9.9, HBM alone 5.6).
+// two exchanges between the blocks (6.5-8.5 us).  Measured, undelayed -> delayed,
+// us a pivot: FP64 1024^2 15.3 -> 9.6, 4096^2 51 -> 36.6 (pass 26.8, its fmas
+// alone 26.8), 8192^2 166 -> 118.1 (pass 108.8, its fmas 107.2); FP32 4096^2
+// 33 -> 8.0, 12288^2 178 -> 16.3.
 #pragma once
 
 #include "tsx_device.cuh"
@@ -68,7 +68,7 @@ struct Delayed {            // one LP and the blocks that work on it
     int* status;            // state word to mark on a timeout (may be null)
     int bt, G;              // this block, blocks
     unsigned smem;          // dynamic shared memory of a block, bytes
-    double eps_d, eps_p;
+    V eps_d, eps_p;         // delay_eps of the tolerances
     long long max_iters;
     int k_cyc, rule;
     long long timeout_ns;
@@ -116,24 +116,57 @@ __device__ __forceinline__ DelayCand delay_none() { return DelayCand{~0ull, INT_
 __device__ __forceinline__ void delay_merge(DelayCand& a, const DelayCand& b, int bland = 0) {
     if (bland ? b.key < a.key : (b.hi < a.hi || (b.hi == a.hi && b.key < a.key))) a = b;
 }
+// The warp's smallest candidate, in every lane: minimum reductions of the
+// value's halves, then of the keys among the lanes that hold them (five
+// shuffle rounds of four words took 0.1 us more).
 __device__ __forceinline__ DelayCand delay_warp(DelayCand a, int bland = 0) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        DelayCand b;
-        b.hi = __shfl_xor_sync(0xffffffffu, a.hi, o);
-        b.key = __shfl_xor_sync(0xffffffffu, a.key, o);
-        b.idx = __shfl_xor_sync(0xffffffffu, a.idx, o);
-        delay_merge(a, b, bland);
+    constexpr unsigned all = 0xffffffffu;
+    bool in = true;
+    if (!bland) {
+        const unsigned h = (unsigned)(a.hi >> 32), l = (unsigned)a.hi;
+        in = h == __reduce_min_sync(all, h);
+        const unsigned x = in ? l : ~0u, y = __reduce_min_sync(all, x);
+        in = in && l == y;
     }
-    return a;
+    const unsigned k = in ? (unsigned)a.key : ~0u;
+    const unsigned m = __reduce_min_sync(all, k);
+    const int from = __ffs(__ballot_sync(all, in && (unsigned)a.key == m)) - 1;
+    DelayCand b;
+    b.hi = __shfl_sync(all, a.hi, from);
+    b.key = (int)m;
+    b.idx = __shfl_sync(all, a.idx, from);
+    return b;
 }
-// dkey as an unsigned number (the order of the doubles is the order of the keys).
+// Values as unsigned keys in their order (dkey; -0 counts as +0): 64 bits of a
+// double, or 32 bits of a float in the upper half, so that the float pivots
+// need no FP64 instruction.
 __device__ __forceinline__ unsigned long long delay_key(double x) {
     return (unsigned long long)dkey(x) ^ 0x8000000000000000ull;
 }
-__device__ __forceinline__ double delay_value(unsigned long long k) {
+__device__ __forceinline__ unsigned long long delay_key(float x) {
+    int b = __float_as_int(x);
+    if (b == INT_MIN) b = 0;
+    b ^= (b >> 31) & 0x7fffffff;
+    return (unsigned long long)((unsigned)b ^ 0x80000000u) << 32;
+}
+template <typename V> __device__ __forceinline__ V delay_value(unsigned long long k);
+template <> __device__ __forceinline__ double delay_value<double>(unsigned long long k) {
     return dkey_value((long long)(k ^ 0x8000000000000000ull));
 }
+template <> __device__ __forceinline__ float delay_value<float>(unsigned long long k) {
+    const int b = (int)((unsigned)(k >> 32) ^ 0x80000000u);
+    return __int_as_float(b ^ ((b >> 31) & 0x7fffffff));
+}
+// The tolerances as values of V: x > eps exactly if x > the largest V not
+// above eps.
+__device__ __forceinline__ void delay_eps(double eps, double& v) { v = eps; }
+__device__ __forceinline__ void delay_eps(double eps, float& v) { v = __double2float_rd(eps); }
+__device__ __forceinline__ bool delay_finite(double x) { return dbits_finite(x); }
+__device__ __forceinline__ bool delay_finite(float x) {
+    return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool delay_nan(double x) { return dbits_nan(x); }
+__device__ __forceinline__ bool delay_nan(float x) { return (__float_as_uint(x) & 0x7fffffffu) > 0x7f800000u; }
 
 template <typename V>
 __device__ __forceinline__ void delay_give_up(const Delayed<V>& D) {
@@ -251,29 +284,61 @@ __device__ __forceinline__ bool delay_barrier(const Delayed<V>& D, DelayScratch&
 // ---------------------------------------------------------- pending chains
 // t through the k pending updates: the entry's own factors at own[u * step]
 // (the multipliers of its row, or the row entries of its column, kept by the
-// block) and the other factors at other[u] (shared memory).
-template <typename V>
-__device__ __forceinline__ V delay_chain(const V* own, int step, const V* other, int k, V t) {
+// block) and the other factors at other[u] (shared memory); both arrays hold K
+// entries, K a multiple of four.  In float a step costs less than a branch:
+// four steps' loads are issued ahead of the four before, and the steps beyond k
+// are computed and dropped (the two chains of a pivot 1.4 -> 0.9 us); a
+// dropped FP64 step would hold the pipe (~80 cycles).
+template <int K>
+__device__ __forceinline__ double delay_chain(const double* own, int step, const double* other, int k, double t) {
 #pragma unroll 4
-    for (int u = 0; u < k; ++u) t = fma_rn(-own[(size_t)u * step], other[u], t);
+    for (int u = 0; u < k; ++u) t = fma_rn(-own[u * step], other[u], t);
+    return t;
+}
+template <int K>
+__device__ __forceinline__ float delay_chain(const float* own, int step, const float* other, int k, float t) {
+    float f[4], r[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        f[x] = own[x * step];
+        r[x] = other[x];
+    }
+#pragma unroll 1
+    for (int u = 0; u < k; u += 4) {
+        const int v = u + 4 < K ? u + 4 : u;
+        float fn[4], rn[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            fn[x] = own[(v + x) * step];
+            rn[x] = other[v + x];
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const float y = fma_rn(-f[x], r[x], t);
+            t = u + x < k ? y : t;
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            f[x] = fn[x];
+            r[x] = rn[x];
+        }
+    }
     return t;
 }
 
-__device__ __forceinline__ bool delay_finite(double x) { return dbits_finite(x); }
-__device__ __forceinline__ bool delay_finite(float x) {
-    return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
-}
-
 // -------------------------------------------------------------- the pass
-// The update tile of a warp: `RS` rows x 32 column groups of 32 bytes, held in
-// registers as four 64-bit words per row and lane (a double, or two floats run
-// by the packed fma.rn.f32x2: one rounding per float, as fmaf).  Per pending
-// pivot a lane takes its 32 bytes of R (shared memory, staged once per column
+// The update tile of a warp: `RS` rows x 1 KB of columns, held in registers as
+// four 64-bit words per row and lane (a double, or two floats run by the packed
+// fma.rn.f32x2: one rounding per float, as fmaf): 16 bytes of each half of the
+// 1 KB, so that a last strip of half the width or less takes half the fused
+// multiply-adds.  Per pending pivot a lane takes its 32 bytes of R (shared memory, staged once per column
 // strip for the whole block) and the rows' multipliers (shared memory, staged
 // per tile, already negated; broadcast reads of two rows at a time).  With one
 // block of 8 warps per SM the next tile's loads are in flight while a tile is
 // updated: 64 KB per SM at any time with 8-row tiles, which is what the HBM
-// stream needs.
+// stream needs.  Four pending pivots per turn of the loop, so that their reads
+// of shared memory overlap (FP32 12288^2: the pass 10.5 -> 8.6 us a pivot; HBM
+// alone 5.6, the fused multiply-adds alone 3.8).
 template <typename V> struct Word;
 template <> struct Word<double> {
     static __device__ __forceinline__ unsigned long long neg(double f) { return __double_as_longlong(-f); }
@@ -304,37 +369,69 @@ __host__ __device__ constexpr size_t delay_smem_bytes(int nt, int rs) {
     return (size_t)kDelayStrips * DelayK<V>::K * 1024 + (size_t)(nt / 32) * DelayK<V>::K * (size_t)(rs * 8 + 16);
 }
 
+// 16-byte accesses, each of a warp's 512 contiguous bytes.  (256-bit ones of
+// four 64-bit words came back from ptxas 13.0 with the last three words not
+// updated in the builds with 128 registers a thread.)
 __device__ __forceinline__ void ld_words(const void* p, unsigned long long* w) {
-    asm volatile("ld.global.L1::no_allocate.v4.b64 {%0,%1,%2,%3}, [%4];"
-                 : "=l"(w[0]), "=l"(w[1]), "=l"(w[2]), "=l"(w[3]) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v2.b64 {%0,%1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(p) : "memory");
 }
 __device__ __forceinline__ void st_words(void* p, const unsigned long long* w) {
-    asm volatile("st.global.v4.b64 [%0], {%1,%2,%3,%4};"
-                 ::"l"(p), "l"(w[0]), "l"(w[1]), "l"(w[2]), "l"(w[3]) : "memory");
+    asm volatile("st.global.v2.b64 [%0], {%1,%2};" ::"l"(p), "l"(w[0]), "l"(w[1]) : "memory");
 }
 
 template <typename V, int RS>
 struct DelayTile {
-    static constexpr int K = DelayK<V>::K, FS = delay_fstride<RS>(), NF = RS * K / 32;
+    static constexpr int K = DelayK<V>::K, FS = delay_fstride<RS>(), NF = RS * K / 32, HALF = 512 / (int)sizeof(V);
     unsigned long long t[RS][4];
     V f[NF];                    // the rows' multipliers, entry lane + 32 x of the RS x K block
-    V* at;                      // the lane's first entry
-    int nrows;                  // 0: the lane's columns lie beyond the tableau
+    V* at;                      // the lane's first entry; the other 16 bytes lie HALF entries on
+    int na, nb;                 // rows to load and store in each half (0: beyond the tableau)
     int strip;                  // staged strip
+    bool wide;                  // the strip has a second half
 
-    __device__ __forceinline__ void load(const Delayed<V>& D, int k, int i0, int col, bool active, int staged) {
+    // left: columns of the tableau from the strip's first on
+    __device__ __forceinline__ void load(const Delayed<V>& D, int k, int i0, int col, int left, int staged) {
+        constexpr int N = 16 / (int)sizeof(V);
         const int lane = threadIdx.x & 31, rows = min(RS, D.m + 1 - i0);
-        at = D.T + (size_t)i0 * (size_t)D.ld + col;
-        nrows = active ? rows : 0;
+        at = D.T + (size_t)i0 * (size_t)D.ld + col + lane * N;
+        na = lane * N < left ? rows : 0;
+        nb = HALF + lane * N < left ? rows : 0;
+        wide = left > HALF;
         strip = staged;
 #pragma unroll
-        for (int r = 0; r < RS; ++r)
-            if (r < nrows) ld_words(at + (size_t)r * (size_t)D.ld, t[r]);
+        for (int r = 0; r < RS; ++r) {
+            if (r < na) ld_words(at + (size_t)r * (size_t)D.ld, t[r]);
+            if (r < nb) ld_words(at + (size_t)r * (size_t)D.ld + HALF, t[r] + 2);
+        }
         const V* fh = D.Fh + (size_t)i0 * K;
 #pragma unroll
         for (int x = 0; x < NF; ++x) {
             const int e = lane + 32 * x;
             f[x] = e / K < rows && e % K < k ? __ldcg(fh + e) : V(0);
+        }
+    }
+    // the first W of the four words of every row
+    template <int W>
+    __device__ __forceinline__ void chain(int k, const unsigned char* rs, const unsigned char* fs) {
+#pragma unroll 4
+        for (int u = 0; u < k; ++u) {
+            const ulonglong2 ra = *reinterpret_cast<const ulonglong2*>(rs + u * 1024);
+            ulonglong2 rb = make_ulonglong2(0, 0);
+            if (W > 2) rb = *reinterpret_cast<const ulonglong2*>(rs + u * 1024 + 512);
+#pragma unroll
+            for (int r = 0; r < RS; r += 2) {
+                const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(fs + u * FS + r * 8);
+                t[r][0] = Word<V>::fma(g.x, ra.x, t[r][0]);
+                t[r][1] = Word<V>::fma(g.x, ra.y, t[r][1]);
+                t[r + 1][0] = Word<V>::fma(g.y, ra.x, t[r + 1][0]);
+                t[r + 1][1] = Word<V>::fma(g.y, ra.y, t[r + 1][1]);
+                if (W > 2) {
+                    t[r][2] = Word<V>::fma(g.x, rb.x, t[r][2]);
+                    t[r][3] = Word<V>::fma(g.x, rb.y, t[r][3]);
+                    t[r + 1][2] = Word<V>::fma(g.y, rb.x, t[r + 1][2]);
+                    t[r + 1][3] = Word<V>::fma(g.y, rb.y, t[r + 1][3]);
+                }
+            }
         }
     }
     __device__ __forceinline__ void update(const Delayed<V>& D, int k, const unsigned char* rs, unsigned char* fs) {
@@ -347,31 +444,20 @@ struct DelayTile {
             *reinterpret_cast<unsigned long long*>(fs + (e % K) * FS + (e / K) * 8) = Word<V>::neg(f[x]);
         }
         __syncwarp();
-#pragma unroll 1
-        for (int u = 0; u < k; ++u) {
-            const ulonglong2 ra = *reinterpret_cast<const ulonglong2*>(rs + u * 1024);
-            const ulonglong2 rb = *reinterpret_cast<const ulonglong2*>(rs + u * 1024 + 512);
+        if (wide)
+            chain<4>(k, rs, fs);
+        else
+            chain<2>(k, rs, fs);
 #pragma unroll
-            for (int r = 0; r < RS; r += 2) {
-                const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(fs + u * FS + r * 8);
-                t[r][0] = Word<V>::fma(g.x, ra.x, t[r][0]);
-                t[r][1] = Word<V>::fma(g.x, ra.y, t[r][1]);
-                t[r][2] = Word<V>::fma(g.x, rb.x, t[r][2]);
-                t[r][3] = Word<V>::fma(g.x, rb.y, t[r][3]);
-                t[r + 1][0] = Word<V>::fma(g.y, ra.x, t[r + 1][0]);
-                t[r + 1][1] = Word<V>::fma(g.y, ra.y, t[r + 1][1]);
-                t[r + 1][2] = Word<V>::fma(g.y, rb.x, t[r + 1][2]);
-                t[r + 1][3] = Word<V>::fma(g.y, rb.y, t[r + 1][3]);
-            }
+        for (int r = 0; r < RS; ++r) {
+            if (r < na) st_words(at + (size_t)r * (size_t)D.ld, t[r]);
+            if (r < nb) st_words(at + (size_t)r * (size_t)D.ld + HALF, t[r] + 2);
         }
-#pragma unroll
-        for (int r = 0; r < RS; ++r)
-            if (r < nrows) st_words(at + (size_t)r * (size_t)D.ld, t[r]);
     }
 };
 
 // Rows 1..m, columns 0..n-1: k pending updates applied to every entry.  Tiles
-// are numbered strip by strip (a strip: 32 column groups); block b takes a
+// are numbered strip by strip (a strip: 1 KB of columns); block b takes a
 // contiguous range of them, so that it stages the pending rows of few strips,
 // and its warps take the range's tiles from a counter.  Two strips are staged
 // at a time: most ranges touch at most two, and a block barrier between strips
@@ -382,14 +468,14 @@ struct DelayTile {
 // AHEAD: the next tile's loads in flight while a tile is updated (needs the
 // registers of one block of 256 threads per SM); without, the other warps of
 // the SM cover a tile's loads.
+// Not inlined: the tile takes most of a thread's registers.
 template <int NT, int RS, bool AHEAD, typename V>
-__device__ __forceinline__ void delay_pass(const Delayed<V>& D, int k, int rev, unsigned char* smem, DelayScratch& s) {
-    constexpr int K = DelayK<V>::K, E = Lanes<V>::E, NS = kDelayStrips;
+__device__ __noinline__ void delay_pass(const Delayed<V>& D, int k, int rev, unsigned char* smem, DelayScratch& s) {
+    constexpr int K = DelayK<V>::K, CS = 1024 / (int)sizeof(V), NS = kDelayStrips;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned char* rs = smem;
     unsigned char* fs = smem + (size_t)NS * K * 1024 + (size_t)w * K * delay_fstride<RS>();
-    const int ngroups = (D.n + E - 1) / E;
-    const int nstrips = (ngroups + 31) / 32;
+    const int nstrips = (D.n + CS - 1) / CS;
     const int ntiles = (D.m + RS - 1) / RS;
     const long long units = (long long)nstrips * ntiles;
     const long long u0 = units * D.bt / D.G, u1 = units * (D.bt + 1) / D.G;
@@ -403,10 +489,10 @@ __device__ __forceinline__ void delay_pass(const Delayed<V>& D, int k, int rev, 
         if (threadIdx.x == 0) s.tile = 0;
         for (int e = threadIdx.x; e < (l - f + 1) * k * 64; e += NT) {
             const int c = e & 63, v = e >> 6, y = v / k, u = v - y * k;   // 16-byte piece c of pivot u, strip f + y
-            const int j = (f + y) * 32 * E + c * (E / 2);
+            const int j = (f + y) * CS + c * (CS / 64);
             if (j < D.ld)
-                *reinterpret_cast<int4*>(rs + (y * K + u) * 1024 + (c & 1) * 512 + (c >> 1) * 16) =
-                    __ldcg(reinterpret_cast<const int4*>(D.Rh + (size_t)u * (size_t)D.ld + j));
+                *reinterpret_cast<ulonglong2*>(rs + (y * K + u) * 1024 + c * 16) =
+                    __ldcg(reinterpret_cast<const ulonglong2*>(D.Rh + (size_t)u * (size_t)D.ld + j));
         }
         __syncthreads();
         const unsigned count = (unsigned)(b - a);
@@ -418,8 +504,7 @@ __device__ __forceinline__ void delay_pass(const Delayed<V>& D, int k, int rev, 
         auto load = [&](DelayTile<V, RS>& tile, unsigned z) {
             const long long unit = rev ? b - 1 - (long long)z : a + (long long)z;
             const int strip = (int)(unit / ntiles), row = (int)(unit - (long long)strip * ntiles);
-            const int g = strip * 32 + lane;
-            tile.load(D, k, 1 + row * RS, g * E, g < ngroups, strip - f);
+            tile.load(D, k, 1 + row * RS, strip * CS, D.n - strip * CS, strip - f);
         };
         unsigned z = next();
         if constexpr (AHEAD) {
@@ -470,6 +555,7 @@ struct DelayOwn {
     V *fo, *ro, *rhs, *obj;
     int* var;
     int fu, fr, ru, rr;
+    V *sf, *sr;   // the pending entries' place in shared memory
     __device__ __forceinline__ DelayOwn(const Delayed<V>& D, unsigned char* smem, size_t pass_bytes) {
         constexpr int K = DelayK<V>::K;
         rper = delay_per(D.m + 1, D.G);
@@ -485,10 +571,22 @@ struct DelayOwn {
         rhs = own ? keep : D.rhs + rb;
         obj = own ? keep + rper : D.T + cb;
         var = own ? reinterpret_cast<int*>(keep + rper + cper) : D.var + cb;
+        sf = reinterpret_cast<V*>(smem);
+        sr = sf + (size_t)rper * K;
         fu = own ? rper : 1;
         fr = own ? 1 : K;
         ru = own ? cper : 1;
         rr = own ? 1 : K;
+    }
+    // the chains of row i (the block's) and of column j; the shared-memory
+    // case apart, so that its loads are shared-memory loads
+    __device__ __forceinline__ V row_chain(int i, const V* other, int k, V t) const {
+        constexpr int K = DelayK<V>::K;
+        return own ? delay_chain<K>(sf + i, rper, other, k, t) : delay_chain<K>(fo + (size_t)i * K, 1, other, k, t);
+    }
+    __device__ __forceinline__ V column_chain(int j, const V* other, int k, V t) const {
+        constexpr int K = DelayK<V>::K;
+        return own ? delay_chain<K>(sr + j, cper, other, k, t) : delay_chain<K>(ro + (size_t)j * K, 1, other, k, t);
     }
 };
 
@@ -510,7 +608,7 @@ __device__ __forceinline__ void delay_begin(const Delayed<V>& D, unsigned char* 
         const int v = __ldcg(D.var + B.cb + j);
         B.obj[j] = x;
         B.var[j] = v;
-        if ((double)x < -D.eps_d) delay_merge(c, DelayCand{delay_key((double)x), v, B.cb + j}, bland);
+        if (x < -D.eps_d) delay_merge(c, DelayCand{delay_key(x), v, B.cb + j}, bland);
     }
     int nf = 0;
     delay_send<NT>(D, D.arg, c, 0, B.cb, B.nc, bland, s);
@@ -537,8 +635,8 @@ template <int NT, typename V, typename Clock>
 __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* smem, size_t pass_bytes, DelayScratch& s,
                                          DelayState& S, Clock& clk) {
     constexpr int K = DelayK<V>::K;
-    static_assert(K <= NT, "one thread per pending pivot");
-    __shared__ V other[K];      // the broadcast factors of a chain
+    static_assert(K <= NT && K % 4 == 0, "one thread per pending pivot, chains by four");
+    __shared__ __align__(16) V other[K];   // the broadcast factors of a chain
     const int t = threadIdx.x;
     const size_t ld = (size_t)D.ld;
     const DelayOwn<V> B(D, smem, pass_bytes);
@@ -550,7 +648,7 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
         // Step 2: the block's rows of column q, up to date; ratios.  The loads
         // that need q are issued together.
         const int q = e.idx, qv = e.key;
-        const double f0 = delay_value(e.hi);   // the objective-row entry of column q
+        const V f0 = delay_value<V>(e.hi);   // the objective-row entry of column q
         V a = V(0);
         if (t < nr) a = __ldcg(D.T + (size_t)(rb + t) * ld + q);
         if (t < k) other[t] = __ldcg(D.RhT + (size_t)q * K + t);
@@ -561,14 +659,14 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
         for (int i = t; i < nr; i += NT) {
             const int row = rb + i;
             if (i != t) a = __ldcg(D.T + (size_t)row * ld + q);
-            a = row == 0 ? (V)f0 : delay_chain(B.fo + (size_t)i * B.fr, B.fu, other, k, a);
+            a = row == 0 ? f0 : B.row_chain(i, other, k, a);
             __stcg(D.Fh + (size_t)row * K + k, a);
             if (B.own) B.fo[(size_t)k * B.fu + i] = a;
             nf |= !delay_finite(a);
-            if (row > 0 && (double)a > D.eps_p) {
-                const double r = (double)div_rn(B.rhs[i], a);
+            if (row > 0 && a > D.eps_p) {
+                const V r = div_rn(B.rhs[i], a);
                 const int key = bland ? __ldcg(D.basis + (row - 1)) : row;
-                if (!dbits_nan(r)) delay_merge(c, DelayCand{delay_key(r), key, row});
+                if (!delay_nan(r)) delay_merge(c, DelayCand{delay_key(r), key, row});
             }
         }
         delay_send<NT>(D, D.rat, c, nf, rb, nr, 0, s);
@@ -578,9 +676,9 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
         clk.lap(3);
         flag |= nf;
         const int p = l.idx;
-        const double theta = delay_value(l.hi);
+        const V theta = delay_value<V>(l.hi);
         if (l.key == INT_MAX) { status = kUnbounded; break; }
-        if (!dbits_finite(theta)) { status = kNumeric; break; }
+        if (!delay_finite(theta)) { status = kNumeric; break; }
         // Step 3, row p: the block's columns up to date, scaled; the objective row
         V* rowp = D.T + (size_t)p * ld + cb;
         V x = V(0);
@@ -599,7 +697,7 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
         }
         // the cycling guard decides the rule of the next Step 1
         if (D.rule == 0) {
-            if (theta <= 0.0) {
+            if (theta <= V(0)) {
                 ++degen;
                 if (D.k_cyc > 0 && degen >= D.k_cyc) bland = 1;
             } else {
@@ -619,7 +717,7 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
                 B.var[j] = leaving;
                 D.var[q] = leaving;
             } else {
-                x = delay_chain(B.ro + (size_t)j * B.rr, B.ru, other, k, x);
+                x = B.column_chain(j, other, k, x);
             }
             const V rj = div_rn(x, piv);
             nf |= !delay_finite(rj);
@@ -627,23 +725,22 @@ __device__ __forceinline__ void delay_round(const Delayed<V>& D, unsigned char* 
             __stcg(D.RhT + (size_t)(cb + j) * K + k, rj);
             __stcg(D.Rh + (size_t)k * ld + cb + j, rj);
             if (B.own) B.ro[(size_t)k * B.ru + j] = rj;
-            ob = fma_rn((V)-f0, rj, ob);
+            ob = fma_rn(-f0, rj, ob);
             B.obj[j] = ob;
-            if ((double)ob < -D.eps_d) delay_merge(c, DelayCand{delay_key((double)ob), B.var[j], cb + j}, bland);
+            if (ob < -D.eps_d) delay_merge(c, DelayCand{delay_key(ob), B.var[j], cb + j}, bland);
         }
         delay_send<NT>(D, D.arg, c, nf, cb, nc, bland, s);
         clk.lap(1);
         // The block's rows, while the candidates travel (visible to the others
         // with the next send): right-hand side; column q starts from zero.
-        const V th = (V)theta;
 #pragma unroll 1
         for (int i = t; i < nr; i += NT) {
             const int row = rb + i;
             if (row == p) {
-                B.rhs[i] = th;
+                B.rhs[i] = theta;
             } else {
                 const V f = B.own ? B.fo[(size_t)k * B.fu + i] : __ldcg(D.Fh + (size_t)row * K + k);
-                B.rhs[i] = fma_rn(-f, th, B.rhs[i]);
+                B.rhs[i] = fma_rn(-f, theta, B.rhs[i]);
                 if (row > 0) __stcg(D.T + (size_t)row * ld + q, V(0));
             }
         }

@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_pe
 // blocks as the blocks of one delayed solve.
 constexpr int kDelayedRows = 8;   // rows of an update tile
 template <int NT, typename V>
-__global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_delayed(Delayed<V> lp, DevState* st) {
+__global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_delayed(Delayed<V> lp, double eps_d, double eps_p, DevState* st) {
     extern __shared__ __align__(128) unsigned char tsx_dyn[];
     __shared__ DelayScratch s;
     __shared__ DelayState S;
@@ -297,6 +297,8 @@ __global__ void __launch_bounds__(NT, persistent_sm_threads(NT) / NT) k_pivot_de
         D = lp;
         D.bt = blockIdx.x;
         D.G = gridDim.x;
+        delay_eps(eps_d, D.eps_d);
+        delay_eps(eps_p, D.eps_p);
         s.passed = 0;
     }
     __syncthreads();

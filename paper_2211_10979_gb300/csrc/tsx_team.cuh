@@ -226,8 +226,8 @@ __device__ bool team_solve_one(const TeamParams<V>& P, const TeamJob<V>& J, Team
         D.bt = bt;
         D.G = (int)C;
         D.smem = smem_bytes;
-        D.eps_d = P.eps_d;
-        D.eps_p = P.eps_p;
+        delay_eps(P.eps_d, D.eps_d);
+        delay_eps(P.eps_p, D.eps_p);
         D.max_iters = P.max_iters < 0 ? 50LL * ((long long)m + n) : P.max_iters;
         D.k_cyc = P.k_cyc;
         D.rule = P.rule;
