@@ -21,6 +21,7 @@
 #include "tsx_host.h"
 #include "tsx_hybrid_host.h"
 #include "tsx_kernels.cuh"
+#include "tsx_lu.cuh"
 #include "tsx_recover.cuh"
 #include "tsx_team.cuh"
 
@@ -1291,11 +1292,118 @@ static lp_status ensure_recovery(lp_handle* h, int k) {
     return LP_OPTIMAL;
 }
 
+// Dynamic shared memory the LU kernels may use (raised to the device's limit
+// once); panel: whether the device can place the panel's cluster.
+struct LuLimits {
+    size_t small_k = 0;
+    bool panel = false;
+};
+static cudaLaunchConfig_t lu_panel_config(cudaStream_t s, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kLuCluster, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kLuCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+static const LuLimits& lu_limits(int device) {
+    static std::once_flag once;
+    static LuLimits lim;
+    std::call_once(once, [device] {
+        int optin = 0;
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+        auto room = [&](const void* kernel) -> size_t {
+            cudaFuncAttributes fa{};
+            if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess || (size_t)optin <= fa.sharedSizeBytes) return 0;
+            const size_t r = (size_t)optin - fa.sharedSizeBytes;
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r) == cudaSuccess ? r
+                                                                                                                  : 0;
+        };
+        lim.small_k = room((const void*)k_rec_lu_small<512>);
+        cudaLaunchAttribute attr[1];
+        cudaLaunchConfig_t cfg = lu_panel_config(nullptr, attr);
+        int clusters = 0;
+        if (cudaFuncSetAttribute((const void*)k_lu_panel<256>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                cudaSuccess &&
+            cudaFuncSetAttribute((const void*)k_lu_update<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)lu_update_smem(256)) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, (const void*)k_lu_panel<256>, &cfg) == cudaSuccess && clusters > 0)
+            lim.panel = true;
+        cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+    });
+    return lim;
+}
+constexpr size_t kLuSharedSm = 100 * 1024;   // shared memory of the small kernel beside other work on its SM
+
+// x_S, y_R and their residuals by LU (tsx_lu.cuh); false (and nothing launched)
+// where the block does not fit: the elimination with the explicit inverse then
+// takes it.  blocks > 0: a share of the GPU beside other launches, one block.
+static lp_status recover_lu(lp_handle* h, const lp_options& o, cudaStream_t s, int k, long long& launches, bool& done) {
+    RecBufs& r = h->rec;
+    const LuLimits& lim = lu_limits(h->device);
+    const size_t cap = o.blocks > 0 ? std::min(lim.small_k, kLuSharedSm) : lim.small_k;
+    done = true;
+    if (k <= kLuSmallMax && lu_small_smem(k) <= cap) {
+        k_rec_lu_small<512><<<1, 512, lu_small_smem(k), s>>>(h->n, h->A, h->b, h->c, r.S, r.Rr, k, r.xS, r.yR, r.rp,
+                                                             r.rd, r.singular);
+        ++launches;
+        CUDA_TRY(cudaGetLastError(), LP_ERR_CUDA);
+        return LP_OPTIMAL;
+    }
+    if (o.blocks > 0 || k > kLuMax || !lim.panel) {
+        done = false;
+        return LP_OPTIMAL;
+    }
+    int nsm = 0, per = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
+    const size_t kk = (size_t)k;
+    double *M = r.M, *U = r.inv, *ip = r.dpiv;
+    int *act = r.pivstep, *piv = r.pivrow;
+    k_rec_gather_square<<<grid_for((long long)(kk * kk), 256, 152 * 16), 256, 0, s>>>(h->n, h->A, r.S, r.Rr, k, M);
+    k_lu_init<<<grid_for(k, 256, 1024), 256, 0, s>>>(k, act);
+    launches += 3;
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = lu_panel_config(s, attr);
+    for (int c0 = 0; c0 < k; c0 += kLuNb) {
+        CUDA_TRY(cudaLaunchKernelEx(&cfg, k_lu_panel<256>, M, U, k, c0, act, piv, ip, r.singular), LP_ERR_CUDA);
+        ++launches;
+        const int rest = k - c0 - kLuNb;
+        if (rest > 0) {
+            // two blocks per SM, each a strip and a share of the row tiles
+            const int x = (rest + 127) / 128, tiles = (rest + 7) / 8;
+            const int y = std::max(1, std::min(tiles, 2 * std::max(1, nsm) / x));
+            k_lu_rows<<<(rest + 31) / 32, 32, 0, s>>>(M, U, k, c0, piv, r.singular);
+            k_lu_update<256><<<dim3(x, y), 256, lu_update_smem(256), s>>>(M, U, k, c0, act, r.singular);
+            ++launches;
+            ++launches;
+        }
+    }
+    CUDA_TRY(cudaGetLastError(), LP_ERR_CUDA);
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_lu_solve<256>, 256, 0), LP_ERR_CUDA);
+    int g = std::max(1, std::min(std::max(1, nsm), grid_for(k, 32, 1 << 20)));
+    if (per < 1) g = 1;
+    int n = h->n, kv = k;
+    const double *A = h->A, *b = h->b, *c = h->c;
+    const int *S = r.S, *R = r.Rr;
+    int* sg = r.singular;
+    DevState* rs = r.rst;
+    long long to = std::max(0LL, o.barrier_timeout_ns);
+    void* args[] = {&n, &A, &b, &c, &S, &R, &kv, &M, &U, &piv, &ip, &r.bR, &r.cS, &r.xS, &r.yR, &r.rp, &r.rd, &sg, &rs, &to};
+    CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_lu_solve<256>, g, 256, args, 0, s), LP_ERR_CUDA);
+    return LP_OPTIMAL;
+}
+
 // Refactorises A_RS for the sets (S, R), solves x_S and y_R (one refinement
 // step), computes the slacks and the objective-row entries, and runs the
-// checks.  Fills `chk`.  Returns LP_ERR_NUMERIC if A_RS is singular.
+// checks; inverse: by the explicit inverse, which cleanup pivots use (set if it
+// was).  Fills `chk`.  Returns LP_ERR_NUMERIC if A_RS is singular.
 static lp_status recover_factor(lp_handle* h, const lp_options& o, cudaStream_t s, const std::vector<int>& S,
-                                const std::vector<int>& R, RecCheck& chk, long long& launches) {
+                                const std::vector<int>& R, RecCheck& chk, long long& launches, bool& inverse) {
     RecBufs& r = h->rec;
     const int m = h->m, n = h->n, k = (int)S.size();
     lp_status st = ensure_recovery(h, k);
@@ -1309,9 +1417,17 @@ static lp_status recover_factor(lp_handle* h, const lp_options& o, cudaStream_t 
     launches += 2;
     int singular = 0;
     if (k > 0) {
-        const size_t kk = (size_t)k;
         CUDA_TRY(cudaMemsetAsync(r.singular, 0, 4, s), LP_ERR_CUDA);
         k_reset_state<<<1, 32, 0, s>>>(r.rst);
+        if (!inverse) {
+            bool done = false;
+            st = recover_lu(h, o, s, k, launches, done);
+            if (st != LP_OPTIMAL) return st;
+            inverse = !done;
+        }
+    }
+    if (k > 0 && inverse) {
+        const size_t kk = (size_t)k;
         int nsm = 0, per = 0, optin = 0;
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
@@ -1384,7 +1500,7 @@ static lp_status recover_factor(lp_handle* h, const lp_options& o, cudaStream_t 
     }
     // slacks s = b - A_:S x_S (every row), objective row d = A_R:^T y_R - c
     k_rec_rows_dot<<<grid_for(32LL * m, 256, 8192), 256, 0, s>>>(m, n, h->A, r.S, k, h->b, -1, r.xS, r.s);
-    k_rec_cols_dot<<<grid_for(n, 256, 8192), 256, 0, s>>>(n, h->A, r.Rr, k, r.yR, -1, h->c, r.d);
+    k_rec_cols_dot<<<grid_for(8LL * n, 256, 8192), 256, 0, s>>>(n, h->A, r.Rr, k, r.yR, -1, h->c, r.d);
     k_rec_check<256><<<1, 256, 0, s>>>(m, n, r.S, r.Rr, k, r.xS, r.s, r.d, r.yR, r.isbasic, r.inR, h->b, h->c,
                                        r.rp, r.rd, r.chk);
     launches += 3;
@@ -1433,12 +1549,17 @@ static lp_status recover(lp_handle* h, const lp_options& o, cudaStream_t s, long
     int cleanup = 0;
     RecCheck chk{};
     lp_status st = LP_OPTIMAL;
+    bool inverse = false;   // the inverse is made once a check has failed
     for (;;) {
-        st = recover_factor(h, o, s, S, R, chk, launches);
+        st = recover_factor(h, o, s, S, R, chk, launches, inverse);
         if (st != LP_OPTIMAL) return st;
         const double pmin = std::min(chk.min_x, chk.min_s);
         const double dmin = std::min(chk.min_d, chk.min_y);
         if (pmin >= -tol && dmin >= -tol) break;                       // optimal in FP64
+        if (!inverse) {
+            inverse = true;
+            continue;
+        }
         if (cleanup >= o.cleanup_max) {
             set_error("lp_solve: FP64 cleanup did not converge in %d pivots", cleanup);
             st = LP_ERR_NUMERIC;
@@ -1453,7 +1574,7 @@ static lp_status recover(lp_handle* h, const lp_options& o, cudaStream_t s, long
             l_kind = structural ? 0 : 1;
             l_at = structural ? chk.min_x_at : chk.min_s_at;
             k_rec_rho<<<grid_for(k, 256, 1024), 256, 0, s>>>(n, h->A, r.S, k, r.inv, l_kind, l_at, r.rho);
-            k_rec_cols_dot<<<grid_for(n, 256, 8192), 256, 0, s>>>(n, h->A, r.Rr, k, r.rho, l_kind == 1 ? l_at : -1,
+            k_rec_cols_dot<<<grid_for(8LL * n, 256, 8192), 256, 0, s>>>(n, h->A, r.Rr, k, r.rho, l_kind == 1 ? l_at : -1,
                                                                   nullptr, r.arow);
             k_rec_dual_ratio<256><<<1, 256, 0, s>>>(n, r.Rr, k, r.arow, r.d, r.isbasic, r.rho, r.yR, 1e-9, r.choice);
             launches += 3;
