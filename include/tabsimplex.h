@@ -161,8 +161,8 @@ typedef struct {
                                      32-byte column group Step 3 updates (read +
                                      write), plus Steps 1-2 and the staging.
                                      Persistent path, condensed: the updates of
-                                     up to 16 (FP32: 32) pivots share one read
-                                     and write of the tableau                   */
+                                     8 to 32 pivots share one read and write of
+                                     the tableau                                */
     int path;                     /* LP_PATH_PERSISTENT, LP_PATH_MULTILAUNCH or
                                      LP_PATH_TEAM (lp_solve_many)               */
     int grid;                     /* blocks of the pivot kernels (team: the

@@ -22,6 +22,7 @@
 #include "tsx_hybrid_host.h"
 #include "tsx_kernels.cuh"
 #include "tsx_lu.cuh"
+#include "tsx_overlap.cuh"
 #include "tsx_recover.cuh"
 #include "tsx_team.cuh"
 
@@ -109,6 +110,8 @@ struct Work {                        // pivot buffers for one precision and layo
     void* RhT = nullptr;
     void* rhs = nullptr;
     DelayRec* recs = nullptr;        // 2 x max_grid
+    Block blk2;                      // overlapped passes: a second copy of the tableau, the rounds' buffers
+    void* T2 = nullptr;
 };
 
 struct RecBufs {                     // FP64 recovery buffers
@@ -343,6 +346,7 @@ static void destroy_impl(lp_handle* h) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     dev_free(h, h->logs);
     dev_free(h, h->work.blk);
+    dev_free(h, h->work.blk2);
     dev_free(h, h->rec.vec);
     dev_free(h, h->rec.kb);
     dev_free(h, h->common);
@@ -586,6 +590,7 @@ static int tableau_ld(int W, int elem) { return (int)align_up((size_t)W, 128 / e
 static lp_status ensure_work(lp_handle* h, int elem, int cond) {
     if (h->work.elem == elem && h->work.cond == cond && h->work.blk.ptr) return LP_OPTIMAL;
     dev_free(h, h->work.blk);
+    dev_free(h, h->work.blk2);
     h->work = Work{};
     const int Ws = cond ? h->n + 1 : h->W;
     const int ld = tableau_ld(Ws, elem);
@@ -756,6 +761,75 @@ static int delayed_grid(int m, int n, int resident, int max_grid, int user_block
     int g = std::min(std::min(resident, max_grid), std::max(1, (std::max(m + 1, n) + 3) / 4));
     if (user_blocks > 0) g = std::min(g, user_blocks);
     return std::max(1, g);
+}
+
+// Overlapped passes (tsx_overlap.cuh): the sizes at which they are faster than
+// passes in turn, where the pass outweighs the longer chains of a pivot.
+// Measured (us a pivot, in turn / overlapped): FP64 1024^2 9.7 / 9.5, 1200^2
+// 11.2 / 9.9, 2049x1531 13.8 / 11.3, 8192^2 117.9 / 111.3; FP32 3000^2 7.5 /
+// 7.9, 4096^2 8.2 / 8.3, 6000^2 9.6 / 9.0, 12288^2 16.4 / 12.2.  Above 4.3 GB
+// the pass is all of a pivot's time and the second copy would only take memory.
+template <typename V>
+static bool overlap_pays(int m, int n) {
+    const double entries = (double)m * (double)n;
+    return entries >= (sizeof(V) == 8 ? 1.0e6 : 2.2e7) && entries * sizeof(V) <= 4.3e9;
+}
+
+// The grid and the second copy for overlapped passes; 0 where they do not fit
+// (the passes then run in turn).  bytes: dynamic shared memory of a block.
+template <typename V>
+static int overlap_ready(lp_handle* h, const lp_options& o, int grid, size_t& bytes) {
+    static std::once_flag once;
+    static size_t limit = 0;
+    const int device = h->device;
+    std::call_once(once, [device] {
+        int optin = 0;
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, k_pivot_overlap<V>) == cudaSuccess && (size_t)optin > fa.sharedSizeBytes &&
+            cudaFuncSetAttribute((const void*)k_pivot_overlap<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 optin - (int)fa.sharedSizeBytes) == cudaSuccess)
+            limit = (size_t)optin - fa.sharedSizeBytes;
+        cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+    });
+    bytes = over_bytes<V>(h->m, h->n, grid);
+    if (bytes > limit) return 0;
+    int nsm = 0, per = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pivot_overlap<V>, kOverNt, bytes) != cudaSuccess ||
+        per * nsm < grid) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (!h->work.blk2.ptr) {
+        const size_t elem = sizeof(V), K = OverK<V>::K;
+        Carve cv;
+        cv.take((size_t)(h->m + 1) * (size_t)h->work.ld * elem);
+        cv.take(2 * (size_t)(h->m + 1) * K * elem);
+        cv.take(2 * (size_t)h->work.ld * K * elem);
+        cv.take(2 * (size_t)h->work.ld * K * elem);
+        if (!dev_alloc_block(h, h->work.blk2, align_up(cv.off, 256))) return 0;
+        h->work.T2 = h->work.blk2.ptr;
+    }
+    return grid;
+}
+
+template <typename V>
+static Overlap<V> overlap_params(lp_handle* h, const Delayed<V>& D) {
+    const size_t elem = sizeof(V), K = OverK<V>::K;
+    Carve cv;
+    cv.take((size_t)(h->m + 1) * (size_t)h->work.ld * elem);
+    const size_t o_F = cv.take(2 * (size_t)(h->m + 1) * K * elem);
+    const size_t o_R = cv.take(2 * (size_t)h->work.ld * K * elem);
+    const size_t o_Rt = cv.take(2 * (size_t)h->work.ld * K * elem);
+    char* base = (char*)h->work.blk2.ptr;
+    Overlap<V> P{};
+    P.D = D;
+    P.D.Fh = (V*)(base + o_F);
+    P.D.Rh = (V*)(base + o_R);
+    P.D.RhT = (V*)(base + o_Rt);
+    P.other = (V*)h->work.T2;
+    return P;
 }
 
 template <int NT, typename V>
@@ -1141,6 +1215,10 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
             dsmem = delayed_smem<NT, V>(m, n, dgrid, dsmem);
         }
     }
+    // ... and the pass of a round may run behind the next round's pivots
+    size_t osmem = 0;
+    const bool over = NT == 256 && dgrid > 0 && o.threads == 0 && overlap_pays<V>(m, n) &&
+                      overlap_ready<V>(h, o, dgrid, osmem) > 0;
     cudaEventRecord(h->ev[0], s);
     k_reset_state<<<1, 32, 0, s>>>(h->st);
     {
@@ -1197,7 +1275,13 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
             DevState* st = h->st;
             void* args[] = {(void*)&D, (void*)&eps_d, (void*)&eps_p, (void*)&st};
             grid_run = dgrid;
-            e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
+            if (over) {
+                Overlap<V> P2 = overlap_params<V>(h, D);
+                void* args2[] = {(void*)&P2, (void*)&eps_d, (void*)&eps_p, (void*)&st};
+                e = cudaLaunchCooperativeKernel((const void*)k_pivot_overlap<V>, dgrid, kOverNt, args2, osmem, s);
+            } else {
+                e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
+            }
         } else {
             e = launch_persistent<NT, V>(P, grid, s);
         }
@@ -1220,6 +1304,7 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     cudaEventRecord(h->ev[2], s);
     CUDA_TRY(cudaMemcpyAsync(&hs, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, s), LP_ERR_CUDA);
     CUDA_TRY(cudaStreamSynchronize(s), LP_ERR_CUDA);
+    if (over && hs.copy) std::swap(h->work.T, h->work.T2);
     path_used = path;
     grid_used = grid_run;
     delayed = dgrid > 0 && path == LP_PATH_PERSISTENT;

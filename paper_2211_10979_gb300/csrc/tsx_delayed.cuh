@@ -174,6 +174,16 @@ __device__ __forceinline__ void delay_give_up(const Delayed<V>& D) {
     if (D.status) atomicCAS(D.status, kRunning, kTimeout);
 }
 
+// Barrier of the block's NT threads (BAR = 0), or of the NT threads that use the
+// named barrier BAR.
+template <int BAR, int NT>
+__device__ __forceinline__ void delay_sync() {
+    if (BAR == 0)
+        __syncthreads();
+    else
+        asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
+}
+
 // An exchange between the D.G blocks: every block sends a candidate, every
 // block gets the smallest.  It is a counted barrier (as grid_barrier_counted)
 // whose arrival also publishes the block's record, so that what a block has
@@ -183,7 +193,7 @@ __device__ __forceinline__ void delay_give_up(const Delayed<V>& D) {
 // records' own stores).
 // cnt: the threads that may hold a candidate; idx0: the block's first row or
 // column.
-template <int NT, typename V>
+template <int NT, int BAR = 0, typename V>
 __device__ __forceinline__ void delay_send(const Delayed<V>& D, DelayRec* recs, DelayCand a, int nonfinite, int idx0,
                                            int cnt, int bland, DelayScratch& s) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -192,7 +202,7 @@ __device__ __forceinline__ void delay_send(const Delayed<V>& D, DelayRec* recs, 
         nonfinite = __any_sync(0xffffffffu, nonfinite);
         if (lane == 0) s.send[w] = DelayPart{a.hi, a.key, a.idx, nonfinite, 0};
     }
-    __syncthreads();
+    delay_sync<BAR, NT>();
     if (threadIdx.x == 0) {
         for (int k = 1; k < NT / 32 && k * 32 < cnt; ++k) {
             const DelayPart x = s.send[k];
@@ -231,7 +241,7 @@ __device__ __forceinline__ bool delay_wait(const Delayed<V>& D, unsigned& passed
 // The smallest candidate of all blocks (every thread returns it); per: rows or
 // columns per block.  False if a wait ran out.  Warp 0 waits, reads the records
 // and reduces them; the others wait at the block barrier.
-template <int NT, typename V>
+template <int NT, int BAR = 0, typename V>
 __device__ __forceinline__ bool delay_gather(const Delayed<V>& D, const DelayRec* recs, int per, int bland,
                                              DelayCand& out, int& nonfinite, DelayScratch& s) {
     if (threadIdx.x < 32) {
@@ -263,21 +273,21 @@ __device__ __forceinline__ bool delay_gather(const Delayed<V>& D, const DelayRec
             s.fail = !ok;
         }
     }
-    __syncthreads();
+    delay_sync<BAR, NT>();
     out = DelayCand{s.got.hi, s.got.key, s.got.idx};
     nonfinite = s.got.nonfinite;
     return s.fail == 0;
 }
 
 // A plain barrier of the D.G blocks on the same counter.
-template <typename V>
+template <int NT, int BAR = 0, typename V>
 __device__ __forceinline__ bool delay_barrier(const Delayed<V>& D, DelayScratch& s) {
-    __syncthreads();
+    delay_sync<BAR, NT>();
     if (threadIdx.x == 0) {
         red_add_release(D.bar_count, 1u);
         s.fail = !delay_wait(D, s.passed);
     }
-    __syncthreads();
+    delay_sync<BAR, NT>();
     return s.fail == 0;
 }
 
@@ -285,10 +295,9 @@ __device__ __forceinline__ bool delay_barrier(const Delayed<V>& D, DelayScratch&
 // t through the k pending updates: the entry's own factors at own[u * step]
 // (the multipliers of its row, or the row entries of its column, kept by the
 // block) and the other factors at other[u] (shared memory); both arrays hold K
-// entries, K a multiple of four.  In float a step costs less than a branch:
-// four steps' loads are issued ahead of the four before, and the steps beyond k
-// are computed and dropped (the two chains of a pivot 1.4 -> 0.9 us); a
-// dropped FP64 step would hold the pipe (~80 cycles).
+// entries.  In float a step costs less than a branch: eight at a time, the steps
+// beyond k computed and dropped; a dropped FP64 step would hold the pipe (~80
+// cycles).
 template <int K>
 __device__ __forceinline__ double delay_chain(const double* own, int step, const double* other, int k, double t) {
 #pragma unroll 4
@@ -297,32 +306,31 @@ __device__ __forceinline__ double delay_chain(const double* own, int step, const
 }
 template <int K>
 __device__ __forceinline__ float delay_chain(const float* own, int step, const float* other, int k, float t) {
-    float f[4], r[4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-        f[x] = own[x * step];
-        r[x] = other[x];
-    }
+    static_assert(K % 8 == 0, "eight steps at a time");
 #pragma unroll 1
-    for (int u = 0; u < k; u += 4) {
-        const int v = u + 4 < K ? u + 4 : u;
-        float fn[4], rn[4];
+    for (int u = 0; u < k; u += 8) {
+        float f[8], r[8];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            fn[x] = own[(v + x) * step];
-            rn[x] = other[v + x];
+        for (int x = 0; x < 8; ++x) {
+            f[x] = own[(u + x) * step];
+            r[x] = other[u + x];
         }
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
+        for (int x = 0; x < 8; ++x) {
             const float y = fma_rn(-f[x], r[x], t);
             t = u + x < k ? y : t;
         }
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            f[x] = fn[x];
-            r[x] = rn[x];
-        }
     }
+    return t;
+}
+// All K pending updates: every load ahead of the chain.
+template <int K, typename V>
+__device__ __forceinline__ V delay_chain_all(const V* own, int step, const V* other, V t) {
+    V f[K];
+#pragma unroll
+    for (int u = 0; u < K; ++u) f[u] = own[u * step];
+#pragma unroll
+    for (int u = 0; u < K; ++u) t = fma_rn(-f[u], other[u], t);
     return t;
 }
 
@@ -379,21 +387,22 @@ __device__ __forceinline__ void st_words(void* p, const unsigned long long* w) {
     asm volatile("st.global.v2.b64 [%0], {%1,%2};" ::"l"(p), "l"(w[0]), "l"(w[1]) : "memory");
 }
 
-template <typename V, int RS>
+template <typename V, int RS, int K>
 struct DelayTile {
-    static constexpr int K = DelayK<V>::K, FS = delay_fstride<RS>(), NF = RS * K / 32, HALF = 512 / (int)sizeof(V);
+    static constexpr int FS = delay_fstride<RS>(), NF = RS * K / 32, HALF = 512 / (int)sizeof(V);
     unsigned long long t[RS][4];
     V f[NF];                    // the rows' multipliers, entry lane + 32 x of the RS x K block
-    V* at;                      // the lane's first entry; the other 16 bytes lie HALF entries on
+    const V* at;                // the lane's first entry; the other 16 bytes lie HALF entries on
     int na, nb;                 // rows to load and store in each half (0: beyond the tableau)
     int strip;                  // staged strip
     bool wide;                  // the strip has a second half
 
     // left: columns of the tableau from the strip's first on
-    __device__ __forceinline__ void load(const Delayed<V>& D, int k, int i0, int col, int left, int staged) {
+    __device__ __forceinline__ void load(const Delayed<V>& D, const V* from, const V* Fh, int k, int i0, int col,
+                                         int left, int staged) {
         constexpr int N = 16 / (int)sizeof(V);
         const int lane = threadIdx.x & 31, rows = min(RS, D.m + 1 - i0);
-        at = D.T + (size_t)i0 * (size_t)D.ld + col + lane * N;
+        at = from + (size_t)i0 * (size_t)D.ld + col + lane * N;
         na = lane * N < left ? rows : 0;
         nb = HALF + lane * N < left ? rows : 0;
         wide = left > HALF;
@@ -403,7 +412,7 @@ struct DelayTile {
             if (r < na) ld_words(at + (size_t)r * (size_t)D.ld, t[r]);
             if (r < nb) ld_words(at + (size_t)r * (size_t)D.ld + HALF, t[r] + 2);
         }
-        const V* fh = D.Fh + (size_t)i0 * K;
+        const V* fh = Fh + (size_t)i0 * K;
 #pragma unroll
         for (int x = 0; x < NF; ++x) {
             const int e = lane + 32 * x;
@@ -434,7 +443,9 @@ struct DelayTile {
             }
         }
     }
-    __device__ __forceinline__ void update(const Delayed<V>& D, int k, const unsigned char* rs, unsigned char* fs) {
+    // shift: from the tableau read to the one written, in entries
+    __device__ __forceinline__ void update(const Delayed<V>& D, ptrdiff_t shift, int k, const unsigned char* rs,
+                                           unsigned char* fs) {
         const int lane = threadIdx.x & 31;
         rs += strip * (K * 1024) + lane * 16;
         __syncwarp();   // the warp has read its previous tile's multipliers
@@ -448,10 +459,11 @@ struct DelayTile {
             chain<4>(k, rs, fs);
         else
             chain<2>(k, rs, fs);
+        V* to = const_cast<V*>(at) + shift;
 #pragma unroll
         for (int r = 0; r < RS; ++r) {
-            if (r < na) st_words(at + (size_t)r * (size_t)D.ld, t[r]);
-            if (r < nb) st_words(at + (size_t)r * (size_t)D.ld + HALF, t[r] + 2);
+            if (r < na) st_words(to + (size_t)r * (size_t)D.ld, t[r]);
+            if (r < nb) st_words(to + (size_t)r * (size_t)D.ld + HALF, t[r] + 2);
         }
     }
 };
@@ -463,16 +475,19 @@ struct DelayTile {
 // at a time: most ranges touch at most two, and a block barrier between strips
 // would leave its last tiles without company (measured at 8192^2 FP64 against
 // one strip and tiles in turn: the wait after the pass 4.5 -> 2.5 us a pivot).
+// from, to: the tableau read and the one written (the same, or two).
 // `rev`: the range backwards (alternate passes start on the tiles the previous
 // one left in L2).
 // AHEAD: the next tile's loads in flight while a tile is updated (needs the
 // registers of one block of 256 threads per SM); without, the other warps of
 // the SM cover a tile's loads.
 // Not inlined: the tile takes most of a thread's registers.
-template <int NT, int RS, bool AHEAD, typename V>
-__device__ __noinline__ void delay_pass(const Delayed<V>& D, int k, int rev, unsigned char* smem, DelayScratch& s) {
-    constexpr int K = DelayK<V>::K, CS = 1024 / (int)sizeof(V), NS = kDelayStrips;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+template <int NT, int RS, bool AHEAD, int K, int BAR = 0, int T0 = 0, typename V>
+__device__ __noinline__ void delay_pass(const Delayed<V>& D, const V* from, V* to, const V* Fh, const V* Rh, int k,
+                                        int rev, unsigned char* smem, DelayScratch& s) {
+    constexpr int CS = 1024 / (int)sizeof(V), NS = kDelayStrips;
+    const int tid = threadIdx.x - T0, lane = tid & 31, w = tid >> 5;
+    const ptrdiff_t shift = to - from;
     unsigned char* rs = smem;
     unsigned char* fs = smem + (size_t)NS * K * 1024 + (size_t)w * K * delay_fstride<RS>();
     const int nstrips = (D.n + CS - 1) / CS;
@@ -485,44 +500,44 @@ __device__ __noinline__ void delay_pass(const Delayed<V>& D, int k, int rev, uns
     for (int x = 0; x < nchunks; ++x) {
         const int f = s0 + (rev ? nchunks - 1 - x : x) * NS, l = min(s1, f + NS - 1);   // strips f..l
         const long long a = max(u0, (long long)f * ntiles), b = min(u1, (long long)(l + 1) * ntiles);
-        __syncthreads();   // the warps are done with the previous strips
-        if (threadIdx.x == 0) s.tile = 0;
-        for (int e = threadIdx.x; e < (l - f + 1) * k * 64; e += NT) {
+        delay_sync<BAR, NT>();   // the warps are done with the previous strips
+        if (tid == 0) s.tile = 0;
+        for (int e = tid; e < (l - f + 1) * k * 64; e += NT) {
             const int c = e & 63, v = e >> 6, y = v / k, u = v - y * k;   // 16-byte piece c of pivot u, strip f + y
             const int j = (f + y) * CS + c * (CS / 64);
             if (j < D.ld)
                 *reinterpret_cast<ulonglong2*>(rs + (y * K + u) * 1024 + c * 16) =
-                    __ldcg(reinterpret_cast<const ulonglong2*>(D.Rh + (size_t)u * (size_t)D.ld + j));
+                    __ldcg(reinterpret_cast<const ulonglong2*>(Rh + (size_t)u * (size_t)D.ld + j));
         }
-        __syncthreads();
+        delay_sync<BAR, NT>();
         const unsigned count = (unsigned)(b - a);
         auto next = [&]() {
             unsigned z = 0;
             if (lane == 0) z = atomicAdd(&s.tile, 1u);
             return __shfl_sync(0xffffffffu, z, 0);
         };
-        auto load = [&](DelayTile<V, RS>& tile, unsigned z) {
+        auto load = [&](DelayTile<V, RS, K>& tile, unsigned z) {
             const long long unit = rev ? b - 1 - (long long)z : a + (long long)z;
             const int strip = (int)(unit / ntiles), row = (int)(unit - (long long)strip * ntiles);
-            tile.load(D, k, 1 + row * RS, strip * CS, D.n - strip * CS, strip - f);
+            tile.load(D, from, Fh, k, 1 + row * RS, strip * CS, D.n - strip * CS, strip - f);
         };
         unsigned z = next();
         if constexpr (AHEAD) {
-            DelayTile<V, RS> cur, ahead;
+            DelayTile<V, RS, K> cur, ahead;
             if (z < count) load(cur, z);
 #pragma unroll 1
             while (z < count) {
                 z = next();
                 if (z < count) load(ahead, z);
-                cur.update(D, k, rs, fs);
+                cur.update(D, shift, k, rs, fs);
                 cur = ahead;
             }
         } else {
 #pragma unroll 1
             for (; z < count; z = next()) {
-                DelayTile<V, RS> tile;
+                DelayTile<V, RS, K> tile;
                 load(tile, z);
-                tile.update(D, k, rs, fs);
+                tile.update(D, shift, k, rs, fs);
             }
         }
     }
@@ -801,16 +816,16 @@ __device__ __forceinline__ void delayed_solve(const Delayed<V>& D, unsigned char
         if (S.status == kDelayFailed) return;
         const int k = S.k;
         if (k > 0) {   // the pending updates applied to the whole tableau, between two barriers
-            if (!delay_barrier(D, s)) break;
+            if (!delay_barrier<NT>(D, s)) break;
             const int rev = (int)(S.passes & 1u);
-            delay_pass<NT, RS, AHEAD>(D, k, rev, smem, s);
+            delay_pass<NT, RS, AHEAD, DelayK<V>::K>(D, D.T, D.T, D.Fh, D.Rh, k, rev, smem, s);
             clk.lap(2);
-            if (!delay_barrier(D, s)) break;
+            if (!delay_barrier<NT>(D, s)) break;
             if (S.flag) {   // 0 x inf in row p: the row again
                 const int cper = delay_per(D.n, D.G), c1 = min(D.n, D.bt * cper + cper);
                 for (int j = D.bt * cper + threadIdx.x; j < c1; j += NT)
                     __stcg(D.T + (size_t)S.last * (size_t)D.ld + j, __ldcg(D.Rh + (size_t)(k - 1) * (size_t)D.ld + j));
-                if (!delay_barrier(D, s)) break;
+                if (!delay_barrier<NT>(D, s)) break;
             }
             if (threadIdx.x == 0) ++S.passes;
             __syncthreads();

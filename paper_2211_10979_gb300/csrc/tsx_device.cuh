@@ -120,6 +120,7 @@ struct DevState {
     unsigned next_slot;                // P4 work counter (slots handed out)
     int fail;                          // delayed updates: a wait ran out
     unsigned passes;                   // delayed updates: passes over the tableau
+    int copy;                          // overlapped passes: the copy that holds the final tableau
     long long phase_ns[6];             // block 0's time per phase: work of
                                        // {select+ratio, stage, update}, then the
                                        // barrier wait after each of them

@@ -36,6 +36,7 @@ __global__ void k_reset_state(DevState* st) {
         st->next_slot = 0;
         st->fail = 0;
         st->passes = 0;
+        st->copy = 0;
         for (int k = 0; k < 6; ++k) st->phase_ns[k] = 0;
     }
 }

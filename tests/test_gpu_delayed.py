@@ -77,3 +77,64 @@ def test_overflow_ends_a_round(tsx, seed, first):   # noqa: F811
         for x, y in zip((one[1].x, one[1].y, one[1].basis, *one[2:5]), (ref[1].x, ref[1].y, ref[1].basis, *ref[2:5])):
             np.testing.assert_array_equal(x, y)
         assert one[1].obj == ref[1].obj or (np.isnan(one[1].obj) and np.isnan(ref[1].obj))
+
+
+# LPs large enough for passes that run behind the pivots (rounds of 8 pivots in
+# FP64): against the oracle, and in FP32 and with overflowing entries against
+# the passes in turn (threads given) and the undelayed path
+@pytest.mark.parametrize("m,n", [(1100, 1000), (2000, 640), (640, 2000)])
+@pytest.mark.parametrize("kw", [{"max_iters": 1}, {"max_iters": 8}, {"max_iters": 9}, {"max_iters": 40}, {},
+                                {"rule": 1, "max_iters": 30}])
+def test_overlapped_passes(tsx, m, n, kw):   # noqa: F811
+    A, b, c = lpgen.dense_lp(m, n, 9)
+    _assert_same(_gpu_run(tsx, A, b, c, path=1, **kw), _oracle_run(A, b, c, **kw))
+
+
+def test_overlapped_passes_revisit_rows_and_columns(tsx):   # noqa: F811
+    # many ties and degenerate pivots: rows and column slots come back within a round
+    rng = np.random.default_rng(4)
+    A = rng.integers(1, 4, (1050, 1000)).astype(float)
+    b = rng.integers(0, 3, 1050).astype(float)
+    c = rng.integers(1, 4, 1000).astype(float)
+    for kw in ({"max_iters": 60}, {"k_cyc": 3, "max_iters": 120}):
+        _assert_same(_gpu_run(tsx, A, b, c, path=1, **kw), _oracle_run(A, b, c, **kw))
+
+
+def test_overlapped_passes_in_float(tsx):   # noqa: F811
+    A, b, c = lpgen.dense_lp(300, 75000, 2)
+    one = _gpu_run(tsx, A, b, c, precision=tsx.LP_PREC_FP32, path=1)
+    ref = _gpu_run(tsx, A, b, c, precision=tsx.LP_PREC_FP32, path=1, threads=256)
+    assert one[5]["iters"] == ref[5]["iters"] > 33
+    for x, y in zip((one[1].x, one[1].y, *one[2:5]), (ref[1].x, ref[1].y, *ref[2:5])):
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("seed,first", [(10, 5), (147, 3), (183, 5), (336, 5)])
+def test_overlapped_passes_overflow(tsx, seed, first):   # noqa: F811
+    rng = np.random.default_rng(seed)
+    A0, b0, c0 = lpgen.dense_lp(20, 15, seed)
+    A0 = A0 - 3.0
+    i = int(rng.integers(20))
+    b0[i] = 0.0
+    A0[i] *= 10.0 ** -rng.integers(290, 308)
+    A0[i][rng.integers(15)] = 5
+    A = np.full((1010, 1000), 1e-3)   # around it: rows that never leave, columns that never enter
+    A[:20, 15:] = 0.0
+    A[:20, :15] = A0
+    b = np.concatenate([b0, np.full(990, 1e6)])
+    c = np.concatenate([c0, np.full(985, -1.0)])
+    for k in (first, -1):
+        one = _gpu_run(tsx, A, b, c, path=1, eps_p=0.0, max_iters=k)
+        ref = _gpu_run(tsx, A, b, c, path=2, eps_p=0.0, max_iters=k)
+        assert not np.isfinite(ref[2]).all()
+        assert one[0] == ref[0] and one[1].iters == ref[1].iters
+        for x, y in zip((one[1].x, one[1].y, one[1].basis, *one[2:5]), (ref[1].x, ref[1].y, ref[1].basis, *ref[2:5])):
+            np.testing.assert_array_equal(x, y)
+
+
+def test_overlapped_passes_time_out(tsx):   # noqa: F811
+    A, b, c = lpgen.dense_lp(1100, 1000, 1)
+    with tsx.Problem(A, b, c) as pr:
+        assert tsx.lp_solve(pr.h, tsx.options(path=1, barrier_timeout_ns=0)) == tsx.LP_ERR_TIMEOUT
+        assert pr.solve(tsx.options(path=1, max_iters=20)) == tsx.LP_ITER_LIMIT
+        np.testing.assert_array_equal(pr.tableau(), _oracle_run(A, b, c, max_iters=20).T)
