@@ -29,7 +29,8 @@
  * pool per device that the library creates and that keeps freed memory for
  * reuse until the process exits).  CUDA events and non-blocking streams that
  * handles no longer need are kept for reuse as well (their creation and
- * destruction serialise concurrent callers in the CUDA runtime).  The pool,
+ * destruction serialise concurrent callers in the CUDA runtime), as are up to
+ * 32 page-locked read-back buffers of 256 KB.  The pool,
  * the events and the streams belong to the device's primary context:
  * resetting the device (cudaDeviceReset) while the library holds them makes
  * later calls fail with LP_ERR_CUDA.

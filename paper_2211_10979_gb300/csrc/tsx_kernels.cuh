@@ -450,6 +450,27 @@ __global__ void k_extract_x(int m, int n, int W, int ld, const V* __restrict__ T
     }
 }
 
+// The whole read-out of a small LP in one launch of one block: the three kernels
+// above one after the other.
+template <typename V>
+__global__ void __launch_bounds__(1024) k_extract_one(int m, int n, int W, int ld, const V* __restrict__ T, int cond,
+                                                      const int* __restrict__ basis, const int* __restrict__ var,
+                                                      double* __restrict__ sol) {
+    const int t = threadIdx.x, nt = blockDim.x;
+    for (int k = t; k < n + m + 1; k += nt)
+        sol[k] = k < n ? 0.0 : k == n + m ? (double)T[W - 1] : cond ? 0.0 : (double)T[k];
+    __syncthreads();
+    if (cond)
+        for (int j = t; j < n; j += nt) {
+            const int v = var[j];
+            if (v >= n) sol[v] = (double)T[j];
+        }
+    for (int i = t; i < m; i += nt) {
+        const int v = basis[i];
+        if (v < n) sol[v] = (double)T[(size_t)(i + 1) * (size_t)ld + (W - 1)];
+    }
+}
+
 // Tableau copy-out widened to double (row-major, W columns).
 template <typename V>
 __global__ void k_widen(int rows, int W, int ld, const V* __restrict__ T, double* __restrict__ out) {
