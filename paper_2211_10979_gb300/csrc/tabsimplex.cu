@@ -1218,7 +1218,7 @@ static lp_status run_hybrid(lp_handle* h, const lp_options& o, cudaStream_t s, c
 // Runs the pivot phase (build + Steps 1-3) on the handle's tableau of V.
 template <int NT, typename V>
 static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, double eps_d, double eps_p,
-                             DevState& hs, long long& launches, int& path_used, int& grid_used, bool& delayed) {
+                             DevState& hs, long long& launches, int& path_used, int& grid_used, int& block_used, bool& delayed) {
     const int m = h->m, n = h->n;
     const int ld = h->work.ld;
     Params<V> P = make_params<V>(m, n, ld, (V*)h->work.T, (V*)h->work.F, (V*)h->work.R, h->work.act,
@@ -1237,6 +1237,14 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     int csize = 0;
     const bool cluster_ok = sizeof(V) == 8 && h->work.cond && (path == LP_PATH_AUTO || path == LP_PATH_CLUSTER);
     if (cluster_ok) csize = cluster_size_for<NT>(h->device, m, n);
+    // Tableau entries of a cluster block.  From 4000 on, 512 threads hide the
+    // update's latencies better (us a pivot, 256 / 512 threads: 100^2 4.1 / 4.2,
+    // 256^2 5.2 / 4.9, 400^2 8.3 / 6.8, 600^2 15.3 / 11.5).  From 15000 on the
+    // whole grid is faster (9.2 whatever the size up to 700^2); LPs up to 600 x
+    // 600, the range the cluster path is documented for, stay on it.
+    const long long centries = csize ? (long long)cluster_rows_per(m, csize) * (n + 1) : 0;
+    const bool cwide = NT == 256 && o.threads == 0 && centries >= 4000;
+    if (path == LP_PATH_AUTO && std::max(m, n) > 600 && centries >= 15000 && coop && coresident > 0) csize = 0;
     if (path == LP_PATH_CLUSTER && !csize) {
         set_error("lp_solve: the cluster path needs an FP64 condensed tableau that fits one cluster's shared memory");
         return LP_ERR_INVALID;
@@ -1308,13 +1316,14 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
         CP.max_iters = o.max_iters;
         CP.k_cyc = o.k_cyc;
         CP.rule = o.rule;
-        cudaError_t e = launch_cluster<NT>(CP, csize, s);
+        cudaError_t e = cwide ? launch_cluster<512>(CP, csize, s) : launch_cluster<NT>(CP, csize, s);
         if (e != cudaSuccess) {
             set_error("lp_solve: cluster launch failed: %s", cudaGetErrorString(e));
             return LP_ERR_CUDA;
         }
         ++launches;
         grid_run = csize;
+        if (cwide) block_used = 512;
     }
     if (path == LP_PATH_PERSISTENT) {
         cudaError_t e = cudaSuccess;
@@ -1331,6 +1340,7 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
                 Overlap<V> P2 = overlap_params<V>(h, D);
                 void* args2[] = {(void*)&P2, (void*)&eps_d, (void*)&eps_p, (void*)&st};
                 e = cudaLaunchCooperativeKernel((const void*)k_pivot_overlap<V>, dgrid, kOverNt, args2, osmem, s);
+                block_used = kOverNt;
             } else {
                 e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
             }
@@ -1807,12 +1817,12 @@ static lp_status solve_nt(lp_handle* h, const lp_options& o, cudaStream_t s) {
     h->final_basis.clear();
     DevState hs{};
     long long launches = 0;
-    int path = 0, grid = 0;
+    int path = 0, grid = 0, block = NT;
     bool delayed = false;
     if (fp32)
-        st = pivot_phase<NT, float>(h, o, s, o.eps_d_fp32, o.eps_p_fp32, hs, launches, path, grid, delayed);
+        st = pivot_phase<NT, float>(h, o, s, o.eps_d_fp32, o.eps_p_fp32, hs, launches, path, grid, block, delayed);
     else
-        st = pivot_phase<NT, double>(h, o, s, o.eps_d, o.eps_p, hs, launches, path, grid, delayed);
+        st = pivot_phase<NT, double>(h, o, s, o.eps_d, o.eps_p, hs, launches, path, grid, block, delayed);
     if (st == LP_ERR_CUDA) return st;
 
     float ms_build = 0.f, ms_pivot = 0.f;
@@ -1842,7 +1852,7 @@ static lp_status solve_nt(lp_handle* h, const lp_options& o, cudaStream_t s) {
     }
     h->stats.path = path;
     h->stats.grid = grid;
-    h->stats.block = NT;
+    h->stats.block = block;
     h->stats.ld = ld;
     h->stats.layout = h->work.cond ? LP_LAYOUT_CONDENSED : LP_LAYOUT_FULL;
     h->stats.precision = o.precision;

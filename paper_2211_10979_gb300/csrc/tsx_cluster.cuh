@@ -22,9 +22,9 @@
 //   - Step 3, pivot row: block r divides its slice of row p (read from the
 //     owner's shared memory) by the pivot element and stores that slice of R
 //     into every block's shared memory;
-//   - cluster barrier; every block updates its rows and its copy of row 0
-//     over one flat index space (full warp instructions), and the new row 0
-//     gives the next entering slot.
+//   - cluster barrier; every block updates its rows over one flat index space
+//     (full warp instructions) and its copy of row 0, and the new row 0 gives
+//     the next entering slot.
 // Two cluster barriers per pivot.  Every value is computed by the same
 // operations as in the other kernels (one IEEE division per R entry and per
 // ratio, one fused multiply-add per updated entry, decisions on the correctly
@@ -36,6 +36,7 @@
 
 #include <cstddef>
 
+#include "tsx_delayed.cuh"
 #include "tsx_select.cuh"
 
 namespace tsx {
@@ -70,18 +71,39 @@ __device__ __forceinline__ void crat_merge(CRat& a, const CRat& b) {
     if (b.rk < a.rk || (b.rk == a.rk && b.key < a.key)) a = b;
 }
 
+// The warp's minimum in every lane: integer minimum reductions find the lane
+// (five shuffle rounds of six words took ~0.15 us more).
 __device__ __forceinline__ CRat warp_crat(CRat a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        CRat b;
-        b.rk = __shfl_xor_sync(0xffffffffu, a.rk, o);
-        b.key = __shfl_xor_sync(0xffffffffu, a.key, o);
-        b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
-        b.a = __shfl_xor_sync(0xffffffffu, a.a, o);
-        b.bvar = __shfl_xor_sync(0xffffffffu, a.bvar, o);
-        crat_merge(a, b);
-    }
-    return a;
+    const DelayCand c = delay_warp(DelayCand{(unsigned long long)a.rk ^ 0x8000000000000000ull, a.key, (int)(threadIdx.x & 31)});
+    CRat b;
+    b.rk = (long long)(c.hi ^ 0x8000000000000000ull);
+    b.key = c.key;
+    b.i = __shfl_sync(0xffffffffu, a.i, c.idx);
+    b.a = __shfl_sync(0xffffffffu, a.a, c.idx);
+    b.bvar = __shfl_sync(0xffffffffu, a.bvar, c.idx);
+    b.pad = 0;
+    return b;
+}
+
+// The entering candidate of the warp under the rule in force, as key (the
+// value; 0 in Bland mode), variable and slot.
+__device__ __forceinline__ DelayCand cluster_entering(const BArg& a, int bland) {
+    return delay_warp(bland ? DelayCand{0, a.fvar, a.fslot}
+                            : DelayCand{(unsigned long long)a.vk ^ 0x8000000000000000ull, a.var, a.slot}, bland);
+}
+
+// x / d, correctly rounded, from y = RN(1 / d): the rounded product, a
+// correction to a faithful quotient, and Markstein's last step (IBM J. Res. Dev.
+// 34, 1990: q + r y rounds correctly for a faithful q, its exact remainder r and
+// the correctly rounded reciprocal y).  Half of a division's latency.  The
+// exponents of x and d keep every intermediate normal; zeros and the rest take
+// the division.
+__device__ __forceinline__ double quotient_rn(double x, double d, double y) {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu, ed = ((unsigned)__double2hiint(d) >> 20) & 0x7ffu;
+    if (ex - 523u > 1000u || ed - 523u > 1000u) return __ddiv_rn(x, d);
+    const double q = x * y;
+    const double f = __fma_rn(__fma_rn(-q, d, x), y, q);
+    return __fma_rn(__fma_rn(-f, d, x), y, f);
 }
 
 // ---- distributed shared memory (sm_90+ cluster PTX) -----------------------
@@ -142,7 +164,8 @@ __host__ __device__ inline size_t cluster_smem_bytes(int m, int n, int C) {
 }
 
 struct ClusterScratch {
-    BArg arg[kMaxWarps];
+    double inv[32];            // reciprocals of the possible pivot elements (up to 32 rows)
+    DelayCand arg[2];          // entering candidates of the objective-row warps
     CRat part;                 // this block's Step 2 result (read remotely)
     CRat merged;               // the cluster's minimum
     int ncand;
@@ -150,7 +173,7 @@ struct ClusterScratch {
 
 template <int NT>
 __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
-    static_assert(NT >= 64, "warp 0 takes the objective row, the others the constraint rows");
+    static_assert(NT >= 96, "warps 0 and 1 take the objective row, the others the constraint rows");
     extern __shared__ __align__(16) unsigned char cl_smem[];
     __shared__ ClusterScratch sc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -182,8 +205,11 @@ __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
     if (warp == 0) {
         BArg a0 = barg_none();
         for (int j = lane; j < n; j += 32) barg_consider_key(a0, Tl[j], var[j], j, epsk);
-        a0 = warp_barg(a0);
-        if (lane == 0) sc.arg[0] = a0;
+        const DelayCand c0 = cluster_entering(a0, P.rule == 1);
+        if (lane == 0) {
+            sc.arg[0] = c0;
+            sc.arg[1] = delay_none();
+        }
     }
     // every block has started before any distributed shared-memory access
     cl_sync();
@@ -192,9 +218,10 @@ __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
     int status = kRunning;
     long long it = 0;
     int bland = P.rule == 1, degen = 0;
-    // the update's flat index space over the own rows 1..nr, warps 1..NW-1
-    constexpr int NU = NT - 32;
-    const int tu = tid - 32;
+    // the update's flat index space over the own rows 1..nr, warps 2..NW-1
+    // (warps 0 and 1: the objective row)
+    constexpr int NU = NT - 64;
+    const int tu = tid - 64;
     const int i_first = 1 + (tu >= 0 ? tu / W1 : 0), j_first = tu >= 0 ? tu - (tu / W1) * W1 : 0;
     const int di = NU / W1, dj = NU - (NU / W1) * W1;
     // block 0's time per phase (thread 0): Step 2, wait at barrier 1, the
@@ -212,10 +239,11 @@ __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
     const int j0 = min(W1, (int)me * sl), j1 = min(W1, j0 + sl);
     while (status == kRunning) {
         // Step 1 (identical in every block): warp 0's result on row 0
-        const BArg a = sc.arg[0];
-        const int qs = bland ? a.fslot : a.slot;
+        DelayCand a = sc.arg[0];
+        delay_merge(a, sc.arg[1], bland);
+        const int qs = a.idx;
         mark(5);
-        if (qs < 0) { status = kOptimal; break; }
+        if (a.key == INT_MAX) { status = kOptimal; break; }
         if (it >= cap) { status = kIterLimit; break; }
         // Step 2 on the own rows.  Up to 32 rows: warp 0 divides every
         // eligible row itself.  More: single-precision screen, then exact
@@ -238,6 +266,13 @@ __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
                 }
                 best = warp_crat(best);
                 if (lane == 0) sc.part = best;
+            } else if (warp == 1) {
+                // the reciprocals of the possible pivot elements, beside the ratios
+                const int l = 1 + lane;
+                if (l <= nr) {
+                    const double av = Tl[(size_t)l * ldc + qs];
+                    if (eligible_bits(av, eps_bits)) sc.inv[lane] = __ddiv_rn(1.0, av);
+                }
             }
         } else {
         if (tid == 0) F[0] = Tl[qs];
@@ -318,9 +353,11 @@ __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
         const unsigned owner = (unsigned)((p - 1) / per);
         const int pl = p - (1 + (int)owner * per) + 1;             // local row of p at its owner
         // Step 3, pivot row: this block's slice of R from row p at the owner
+        // (the owner has the pivot's reciprocal where every block has up to 32 rows)
         for (int j = j0 + tid; j < j1; j += NT) {
             const double v = cl_ld_f64(cl_map(smem_addr(Tl + (size_t)pl * ldc + j), owner));
-            R[j] = __ddiv_rn(j == qs ? 1.0 : v, piv);   // one division, whichever operand
+            const double x = j == qs ? 1.0 : v;
+            R[j] = per <= 32 ? quotient_rn(x, piv, cl_ld_f64(cl_map(smem_addr(sc.inv + pl - 1), owner))) : __ddiv_rn(x, piv);
         }
         __syncthreads();
         for (int t = tid; t < (j1 - j0) * (int)C; t += NT) {
@@ -355,20 +392,21 @@ __global__ void __launch_bounds__(NT) k_cluster_solve(ClusterParams P) {
         // Step 3, update of row 0 and the own rows over one flat index space;
         // the owner's row p becomes R
         const int plocal = owner == me ? pl : -1;
-        __syncthreads();   // var[qs] is read by the objective-row candidates
-        if (warp == 0) {
-            // row 0 and the next Step 1
+        if (warp < 2) {
+            // row 0 and the next Step 1 (var[qs] may still be changing), two
+            // warps, three entries of a lane in flight
             BArg an = barg_none();
             const double f0 = F[0];
-            for (int j = lane; j < W1; j += 32) {
+#pragma unroll 3
+            for (int j = tid; j < W1; j += 64) {
                 const double v = __fma_rn(-f0, R[j], j == qs ? 0.0 : Tl[j]);
                 Tl[j] = v;
-                if (j < n) barg_consider_key(an, v, var[j], j, epsk);
+                if (j < n) barg_consider_key(an, v, j == qs ? best.bvar : var[j], j, epsk);
             }
-            an = warp_barg_rule(an, bland);   // the next Step 1 reads these fields only
-            if (lane == 0) sc.arg[0] = an;
+            const DelayCand cn = cluster_entering(an, bland);
+            if (lane == 0) sc.arg[warp] = cn;
         } else {
-            // the own constraint rows, flat over warps 1..NW-1
+            // the own constraint rows, flat over warps 2..NW-1
             flat_update(Tl, ldc, nr, W1, n, F, R, qs, plocal, var, epsk, i_first, j_first, di, dj);
         }
         __syncthreads();
