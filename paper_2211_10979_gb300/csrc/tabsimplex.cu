@@ -1961,6 +1961,16 @@ static bool team_takes(int device, int m, int ld, int elem, int C) {
     return ((size_t)ld + delay_per(m + 1, C)) * elem <= (size_t)std::max(0, optin);
 }
 
+// FP64 LPs whose update keeps the whole grid's FP64 pipes busy (from 4e6 entries
+// on, a pass of 6.7 us a pivot) are faster one at a time than on a team that
+// outlasts the others.  96 LPs with m, n log-uniform in [180, 3000], three sets
+// of data, ms a call: never 67 / 96 / 89, from 2.5e6 80 / 80 / 76, from 4e6
+// 72 / 73 / 69, from 6e6 76 / 74 / 66 (the fused multiply-adds alone 43-46).
+template <typename V>
+static bool grid_fills(int m, int n) {
+    return sizeof(V) == 8 && (double)m * (double)n >= 4.0e6;
+}
+
 template <typename V>
 static TeamJob<V> team_job(const lp_handle* h) {
     TeamJob<V> J{};
@@ -2078,7 +2088,8 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
     size_t smem = pass_bytes;
     for (int k = 0; k < count; ++k) {
         lp_handle* h = hs[k];
-        if (!team_takes(device, h->m, h->work.ld, elem, C)) {
+        if (!team_takes(device, h->m, h->work.ld, elem, C) ||
+            (o.blocks == 0 && reserve_blocks == 0 && grid_fills<V>(h->m, h->n))) {
             alone.push_back(k);
             continue;
         }

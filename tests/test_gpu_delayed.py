@@ -138,3 +138,22 @@ def test_overlapped_passes_time_out(tsx):   # noqa: F811
         assert tsx.lp_solve(pr.h, tsx.options(path=1, barrier_timeout_ns=0)) == tsx.LP_ERR_TIMEOUT
         assert pr.solve(tsx.options(path=1, max_iters=20)) == tsx.LP_ITER_LIMIT
         np.testing.assert_array_equal(pr.tableau(), _oracle_run(A, b, c, max_iters=20).T)
+
+
+def test_many_with_a_large_lp(tsx):   # noqa: F811
+    # above 4e6 entries an FP64 LP of a list is solved on the whole grid
+    shapes = [(300, 200), (2100, 1950), (700, 300)]
+    problems = [lpgen.dense_lp(m, n, 20 + k) for k, (m, n) in enumerate(shapes)]
+    refs = [oracle.solve(*p) for p in problems]
+    for blocks, large in ((0, tsx.LP_PATH_PERSISTENT), (16, tsx.LP_PATH_TEAM)):
+        prs = [tsx.Problem(*p) for p in problems]
+        try:
+            assert tsx.solve_many(prs, tsx.options(blocks=blocks)) == [r.status for r in refs]
+            for pr, ref, path in zip(prs, refs, (tsx.LP_PATH_TEAM, large, tsx.LP_PATH_TEAM)):
+                sol = pr.solution()
+                assert sol.iters == ref.iters and sol.obj == ref.obj and pr.stats()["path"] == path
+                np.testing.assert_array_equal(sol.x, ref.x)
+                np.testing.assert_array_equal(sol.y, ref.y)
+        finally:
+            for pr in prs:
+                pr.close()
