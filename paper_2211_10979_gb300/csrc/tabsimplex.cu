@@ -697,8 +697,9 @@ static size_t persistent_smem() {
 
 // Rows of an update slot of the persistent kernel for an LP with m rows:
 // persistent_rows(NT), or 8 below 3072 rows, where 16-row slots are too few
-// to spread evenly over the grid's warps (measured against 16: 1024² +17 %,
-// 2048² +2.5 %, 4096² -3 %).
+// to spread evenly over the grid's warps (measured against 16 with one update
+// per pivot on condensed tableaux, which the delayed kernels solve by now; the
+// full layout's slots are the same: 1024² +17 %, 2048² +2.5 %, 4096² -3 %).
 template <int NT>
 static int persistent_slot_rows(int m) {
     return persistent_rows(NT) > 8 && m < 3072 ? 8 : persistent_rows(NT);
@@ -2270,7 +2271,10 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
 // one has ended (teams exit after idle_ns without work).
 namespace {
 constexpr unsigned kLaneCap = 4096;               // ring entries per list
-constexpr long long kLaneIdleNs = 2'000'000;      // the teams exit 2 ms after the last one's work
+// The teams exit 5 ms after the last one's work.  A new launch waits for the
+// kernels that took its SMs meanwhile (a recovery of a few ms), and small LPs
+// queue behind it: at 2000 LPs/s, 2 ms gives 16 launches a second, 5 ms under 1.
+constexpr long long kLaneIdleNs = 5'000'000;
 constexpr long long kLaneIdleCapNs = 10'000'000'000LL;   // bound on one team's wait for work
 constexpr double kLaneHeavyWork = 1.5e10;         // (m+1) (n+1) (m+n) above this: the wide teams' list
 }

@@ -9,8 +9,9 @@
 // (FP32: 32) pivots share one pass over the tableau.  The arithmetic and the
 // tie rules are those of the single-LP kernels, so every pivot and value equals
 // lp_solve's.  Measured against one update per pivot (bound by HBM, 0.86 of
-// it): 96 FP64 LPs with m, n log-uniform in [180, 3000] 110-118 -> 63-87 ms (two
-// boxes), a burst of 200 FP32 requests with m, n in [32, 4096] 201 -> 71 ms.
+// it): 96 FP64 LPs with m, n log-uniform in [180, 3000] 114 -> 85 ms a call (79
+// with those of 4e6 entries or more solved on the whole grid), a burst of 200
+// FP32 requests with m, n in [32, 4096] 201 -> 71 ms.
 #pragma once
 
 #include "tsx_delayed.cuh"
@@ -313,10 +314,16 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(Tea
 //     system scope), which the host polls;
 //   - a team that finds nothing to claim keeps polling while another team
 //     still works (a job published meanwhile is taken at once); once no team
-//     has had work for idle_ns (or the stop word is set) every team exits, and
-//     the host starts a new launch when jobs are waiting and none runs.  Every
-//     wait is bounded: the claim loop by idle_cap_ns and a spin cap, the team
-//     barriers as in k_team_solve (a team that gives up clears its busy mark).
+//     has had work for idle_ns one of them closes the launch, every team exits,
+//     and the host starts a new launch when jobs are waiting and none runs.
+//     Closing is a bit of the busy word, set by a compare-and-swap from zero,
+//     and a team marks itself busy before it claims: a launch never goes on
+//     with some of its teams gone.  (When each team left on its own clock, one
+//     that claimed a job just then kept the launch alive alone, and the stream
+//     behind it waited for that team: 7 s at 2000 LPs/s.)  Every wait is
+//     bounded: the claim loop by idle_cap_ns and a spin cap, after which the
+//     launch closes as well, the team barriers as in k_team_solve (a team that
+//     gives up clears its busy mark and closes the launch).
 // ---------------------------------------------------------------------------
 template <typename V>
 struct ServeRing {
@@ -332,11 +339,13 @@ struct TeamServeParams {
     ServeRing<V> ring;
     unsigned cap;              // entries per list, a power of two
     unsigned* head;            // device memory: jobs claimed per list [2]
-    unsigned* busy;            // device memory: teams solving a job (zero at launch)
+    unsigned* busy;            // device memory: teams solving a job (zero at launch) and kServeClosed
     TeamJob<V>* jcopy;         // device memory: per team, the job it solves
     long long idle_ns;         // every team leaves once none has had work for this long
     long long idle_cap_ns;     // bound on a team's wait while others still work
 };
+
+constexpr unsigned kServeClosed = 0x80000000u;   // no further job is claimed in this launch
 
 __device__ __forceinline__ unsigned ld_acquire_sys(const unsigned* p) {
     unsigned v;
@@ -368,11 +377,16 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
                 (unsigned long long)(P.idle_cap_ns > 0 ? P.idle_cap_ns : 0) / 500ull + 64ull;
             long long t_idle = t0;   // since when no team has been seen working
             for (unsigned long long spins = 0;; ++spins) {
-                for (int pass = 0; pass < 2 && got < 0; ++pass) {
+                bool marked = false, closed = false;
+                for (int pass = 0; pass < 2 && got < 0 && !closed; ++pass) {
                     const int l = pass == 0 ? li : 1 - li;
                     const unsigned tl = ld_acquire_sys(P.ring.tail + l);
                     unsigned h = *(volatile unsigned*)(P.head + l);
-                    while ((int)(tl - h) > 0) {
+                    if ((int)(tl - h) > 0 && !marked) {
+                        marked = true;
+                        closed = (atomicAdd(P.busy, 1u) & kServeClosed) != 0u;
+                    }
+                    while (!closed && (int)(tl - h) > 0) {
                         const unsigned prev = atomicCAS(P.head + l, h, h + 1u);
                         if (prev == h) {
                             got = l;
@@ -382,15 +396,18 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
                         h = prev;
                     }
                 }
-                if (got >= 0) {
-                    atomicAdd(P.busy, 1u);
+                if (got >= 0) break;
+                if (marked) atomicSub(P.busy, 1u);
+                const long long now = global_ns();
+                const unsigned busy = *(volatile unsigned*)P.busy;
+                if (closed || (busy & kServeClosed)) break;
+                if (busy != 0u) t_idle = now;
+                if (ld_acquire_sys(P.ring.stop) != 0u) break;
+                if (now - t_idle >= P.idle_ns && atomicCAS(P.busy, 0u, kServeClosed) == 0u) break;
+                if (now - t0 >= P.idle_cap_ns || spins >= max_spins) {
+                    atomicOr(P.busy, kServeClosed);
                     break;
                 }
-                const long long now = global_ns();
-                if (*(volatile unsigned*)P.busy != 0u) t_idle = now;
-                if (ld_acquire_sys(P.ring.stop) != 0u || now - t_idle >= P.idle_ns || now - t0 >= P.idle_cap_ns ||
-                    spins >= max_spins)
-                    break;
                 __nanosleep(500);
             }
             if (got >= 0) {
@@ -432,7 +449,10 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
             st->phase_ns[0] = global_ns();
         }
         if (!team_solve_one<NT>(P.tp, s.job, ts, bt, C, tsx_dyn, smem_bytes, s)) {
-            if (bt == 0 && threadIdx.x == 0) atomicSub(P.busy, 1u);
+            if (bt == 0 && threadIdx.x == 0) {
+                atomicOr(P.busy, kServeClosed);
+                atomicSub(P.busy, 1u);
+            }
             return;
         }
         if (bt == 0 && threadIdx.x == 0) {

@@ -195,6 +195,27 @@ def test_request_admitted_into_running_work_finishes_first(tsx):
         np.testing.assert_array_equal(r.y, alone.y)
 
 
+@pytest.mark.parametrize("pause", [0.0, 0.004, 0.005, 0.02])
+def test_bursts_around_the_idle_limit(tsx, pause):
+    # the team launch closes once no team has had work for 5 ms: bursts that
+    # arrive just before, at and after that moment are all solved, by the
+    # running launch or the next one
+    A, b, c = lpgen.dense_lp(300, 260, 33)
+    st1, alone = _alone_fp32(tsx, A, b, c)
+    assert st1 == tsx.LP_OPTIMAL
+    with tsx.Server(workers=4) as sv:
+        for _ in range(12):
+            tickets = [sv.submit(A, b, c) for _ in range(20)]
+            for t in tickets:
+                assert sv.wait(t, 60.0) == tsx.LP_OPTIMAL
+                r = sv.result(t)
+                assert r.obj == alone.obj and r.iters == alone.iters
+                np.testing.assert_array_equal(r.x, alone.x)
+            time.sleep(pause)
+        st = sv.stats()
+    assert st["lane_lps"] == 240 and st["lane_launches"] >= (12 if pause >= 0.02 else 1)
+
+
 @pytest.mark.parametrize("continuous", [1, 0])
 def test_invalid_device_request_in_a_wave(tsx, continuous):
     # device inputs are checked in the team kernel's build: a request with
