@@ -90,7 +90,9 @@ typedef struct {
                                      one thread-block cluster's shared memory
                                      (up to 16 blocks, about 227 KB each: the
                                      whole solve on chip, two cluster barriers
-                                     per pivot), else the persistent
+                                     per pivot) and has at most 600 rows and
+                                     columns or less than 15000 entries per
+                                     block, else the persistent
                                      cooperative kernel when it can be
                                      launched, else one launch per phase;
                                      LP_PATH_PERSISTENT, LP_PATH_MULTILAUNCH or
@@ -108,7 +110,8 @@ typedef struct {
                                      columns whose scaled pivot row entries are
                                      all zero (their update is the identity);
                                      0: update every column                     */
-    int threads;                  /* threads per block, 0 = default (256)       */
+    int threads;                  /* threads per block, 0 = default (256; 512
+                                     for large LPs and large cluster blocks)    */
     int blocks;                   /* grid size cap, 0 = all co-resident blocks
                                      (lp_solve_many: blocks per team)           */
     long long log_capacity;       /* pivots whose (q, p) pair is recorded;
@@ -164,7 +167,8 @@ typedef struct {
                                      Persistent path, condensed: the updates of
                                      8 to 32 pivots share one read and write of
                                      the tableau                                */
-    int path;                     /* LP_PATH_PERSISTENT, LP_PATH_MULTILAUNCH or
+    int path;                     /* LP_PATH_PERSISTENT, LP_PATH_MULTILAUNCH,
+                                     LP_PATH_CLUSTER, LP_PATH_HYBRID or
                                      LP_PATH_TEAM (lp_solve_many)               */
     int grid;                     /* blocks of the pivot kernels (team: the
                                      narrow team size)                          */

@@ -40,7 +40,7 @@ def _deps():
 # Sources of the single-LP pivot kernels' device code (a profile of the
 # persistent kernel stays valid while these are unchanged and the launch
 # shape recorded with it is the same).
-PIVOT_SOURCES = ("tsx_delayed.cuh", "tsx_device.cuh", "tsx_kernels.cuh")
+PIVOT_SOURCES = ("tsx_delayed.cuh", "tsx_device.cuh", "tsx_kernels.cuh", "tsx_overlap.cuh")
 
 
 def source_digest(names=None) -> str:

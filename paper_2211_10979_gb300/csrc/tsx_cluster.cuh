@@ -4,9 +4,9 @@
 // processors, here over the C <= 16 SMs of one cluster).
 //
 // For LPs whose pivots are too small to fill the GPU, the cost of a pivot on
-// the grid-wide kernel is its fixed part: three device-wide barriers through
-// L2 and the reductions' round trips (~20 us at m = n = 256, where the update
-// itself moves 1 MB).  Here a cluster of C blocks keeps the tableau on chip
+// the grid-wide kernel is its fixed part: two device-wide exchanges through L2
+// and the chains between them (~9 us whatever the size up to 700 x 700; here
+// 4.9 at m = n = 256).  Here a cluster of C blocks keeps the tableau on chip
 // and synchronises with the hardware cluster barrier:
 //   - block r owns constraint rows [g0, g1) of the condensed tableau (the n
 //     nonbasic columns plus the right-hand side, var[] giving each slot's

@@ -283,8 +283,8 @@ __device__ __forceinline__ RatPart rat_none() { return RatPart{__longlong_as_dou
 // variable: the column index itself in the full tableau, var[] in the
 // condensed one.
 // Merges of Step 1-2 partials (shuffle trees, block and grid reductions)
-// compare keys: measured 5888 vs 5817 pivots/s at 8192^2 (the ratio and
-// staging phases 2 us shorter per pivot).  Keys in the per-entry candidate
+// compare keys: measured 5888 vs 5817 pivots/s at 8192^2 with one update per
+// pivot (the ratio and staging phases 2 us shorter per pivot).  Keys in the per-entry candidate
 // scans as well cost more ALU work in the objective-row pass than the FP64
 // comparisons they replace (5709).
 #ifndef TSX_KEYS

@@ -248,7 +248,6 @@ __global__ void __launch_bounds__(NT) k_rec_lu_small(int n, const double* __rest
 // ------------------------------------------------------------- large k
 constexpr int kLuNb = 32;        // columns of a panel
 constexpr int kLuCluster = 16;   // blocks of the panel cluster
-constexpr int kLuPld = kLuNb + 1;
 
 struct LuCand {
     unsigned long long key;
