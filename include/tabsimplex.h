@@ -254,7 +254,8 @@ lp_status lp_solve(lp_t h, const lp_options *opt);
  *   status   HOST output, count entries: each LP's status as lp_solve returns it
  * An LP whose pivot row and row multipliers would not fit one block's shared
  * memory is solved by lp_solve after the launch (it fills the GPU by itself),
- * and so is, with blocks = 0, an FP64 LP of 4e6 tableau entries or more.  Afterwards each handle
+ * and so is, with blocks = 0, an FP64 LP of 4e6 tableau entries or more that
+ * would outlast the rest of the list on a team.  Afterwards each handle
  * answers lp_get_solution, lp_get_tableau and lp_get_stats as after lp_solve
  * (stats.path = LP_PATH_TEAM, stats.pivot_ms = the whole launch, no pivot
  * log).  Returns LP_OPTIMAL when the call ran (per-LP outcomes in status), or

@@ -1963,13 +1963,16 @@ static bool team_takes(int device, int m, int ld, int elem, int C) {
 }
 
 // FP64 LPs whose update keeps the whole grid's FP64 pipes busy (from 4e6 entries
-// on, a pass of 6.7 us a pivot) are faster one at a time than on a team that
-// outlasts the others.  96 LPs with m, n log-uniform in [180, 3000], three sets
-// of data, ms a call: never 67 / 96 / 89, from 2.5e6 80 / 80 / 76, from 4e6
-// 72 / 73 / 69, from 6e6 76 / 74 / 66 (the fused multiply-adds alone 43-46).
+// on, a pass of 6.7 us a pivot) and that would outlast the list on a wide team
+// are faster alone on the grid: work is the LP's, wide what the wide team of 4 C
+// blocks gets through while the grid does the whole list.  Geometric means in
+// ms a call, never / all from 4e6 on / those above 0.25, 0.35, 0.5 of wide: three
+// lists of 96 LPs with m, n log-uniform in [180, 3000] 83 / 67 / 67, 67, 76; eight
+// other lists 62 / 56 / 56, 54, 54.  Lists of the first kind that a team launch
+// packs well by chance lose up to 10 % (54 / 62 / 60, 59, 58).
 template <typename V>
-static bool grid_fills(int m, int n) {
-    return sizeof(V) == 8 && (double)m * (double)n >= 4.0e6;
+static bool grid_fills(int m, int n, double work, double wide) {
+    return sizeof(V) == 8 && (double)m * (double)n >= 4.0e6 && work > 0.35 * wide;
 }
 
 template <typename V>
@@ -2087,16 +2090,21 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
     std::vector<double> work;
     const size_t pass_bytes = delay_smem_bytes<V>(NT, kTeamRows);
     size_t smem = pass_bytes;
+    // an LP's share of the list: entries times the m + n estimate of its pivots
+    auto lp_work = [](const lp_handle* h) { return (double)(h->m + 1) * h->work.ld * (double)(h->m + h->n); };
+    double wide = 0.0;
+    for (int k = 0; k < count; ++k) wide += lp_work(hs[k]);
+    wide *= 4.0 * C / ((double)(team_sm_threads(NT) / NT) * nsm);
     for (int k = 0; k < count; ++k) {
         lp_handle* h = hs[k];
         if (!team_takes(device, h->m, h->work.ld, elem, C) ||
-            (o.blocks == 0 && reserve_blocks == 0 && grid_fills<V>(h->m, h->n))) {
+            (o.blocks == 0 && reserve_blocks == 0 && grid_fills<V>(h->m, h->n, lp_work(h), wide))) {
             alone.push_back(k);
             continue;
         }
         jobs.push_back(team_job<V>(h));
         who.push_back(k);
-        work.push_back((double)(h->m + 1) * h->work.ld * (double)(h->m + h->n));
+        work.push_back(lp_work(h));
         smem = std::max(smem, delay_own_bytes<V>(h->m, h->n, C, pass_bytes));
     }
     smem = std::min(smem, smem_limit);

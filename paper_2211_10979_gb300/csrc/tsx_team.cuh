@@ -9,8 +9,8 @@
 // (FP32: 32) pivots share one pass over the tableau.  The arithmetic and the
 // tie rules are those of the single-LP kernels, so every pivot and value equals
 // lp_solve's.  Measured against one update per pivot (bound by HBM, 0.86 of
-// it): 96 FP64 LPs with m, n log-uniform in [180, 3000] 114 -> 85 ms a call (79
-// with those of 4e6 entries or more solved on the whole grid), a burst of 200
+// it): 96 FP64 LPs with m, n log-uniform in [180, 3000] 114 -> 85 ms a call (67-79
+// with the largest solved on the whole grid), a burst of 200
 // FP32 requests with m, n in [32, 4096] 201 -> 71 ms.
 #pragma once
 

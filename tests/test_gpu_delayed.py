@@ -141,7 +141,8 @@ def test_overlapped_passes_time_out(tsx):   # noqa: F811
 
 
 def test_many_with_a_large_lp(tsx):   # noqa: F811
-    # above 4e6 entries an FP64 LP of a list is solved on the whole grid
+    # an FP64 LP above 4e6 entries that would outlast its list is solved on the
+    # whole grid
     shapes = [(300, 200), (2100, 1950), (700, 300)]
     problems = [lpgen.dense_lp(m, n, 20 + k) for k, (m, n) in enumerate(shapes)]
     refs = [oracle.solve(*p) for p in problems]
@@ -157,3 +158,25 @@ def test_many_with_a_large_lp(tsx):   # noqa: F811
         finally:
             for pr in prs:
                 pr.close()
+
+
+@pytest.mark.parametrize("count,on_grid", [(14, False), (13, True)])
+def test_many_large_lps_by_their_share(tsx, count, on_grid):   # noqa: F811
+    # equal LPs above 4e6 entries: each is 1 / count of the list, and goes to the
+    # grid where that is above 0.35 of what a wide team (64 of 304 blocks) gets
+    # through meanwhile, 0.0737 of it
+    A, b, c = lpgen.dense_lp(2050, 1960, 40)
+    prs = [tsx.Problem(A, b, c) for _ in range(count)]
+    try:
+        assert prs[0].solve() == tsx.LP_OPTIMAL
+        alone = prs[0].solution()
+        assert tsx.solve_many(prs) == [tsx.LP_OPTIMAL] * count
+        for pr in prs:
+            assert pr.stats()["path"] == (tsx.LP_PATH_PERSISTENT if on_grid else tsx.LP_PATH_TEAM)
+            sol = pr.solution()
+            assert sol.iters == alone.iters and sol.obj == alone.obj
+            np.testing.assert_array_equal(sol.x, alone.x)
+            np.testing.assert_array_equal(sol.y, alone.y)
+    finally:
+        for pr in prs:
+            pr.close()
