@@ -1366,6 +1366,10 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     }
     cudaEventRecord(h->ev[2], s);
     CUDA_TRY(read_back(&hs, h->st, sizeof(DevState), s), LP_ERR_CUDA);
+    // Delayed updates: a block that gave up has not stored its parts of the
+    // result, also where block 0, whose waits all ended in time, has written a
+    // final status (nothing orders the two; the team kernel has a barrier there).
+    if (hs.fail) hs.status = kTimeout;
     if (over && hs.copy) std::swap(h->work.T, h->work.T2);
     path_used = path;
     grid_used = grid_run;

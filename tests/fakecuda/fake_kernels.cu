@@ -1,0 +1,62 @@
+// The kernels as far as the fake runtime plays them: the state words, the final
+// basis and the lane's rings, from the library's own structs.
+#include <cuda_runtime.h>
+
+#include <cstring>
+
+#include "tsx_cluster.cuh"
+#include "tsx_device.cuh"
+#include "tsx_team.cuh"
+
+extern "C" {
+int fake_plan_status = 0, fake_plan_fail = 0, fake_plan_k = 0;
+}
+
+namespace {
+using tsx::DevState;
+bool is(const char* name, const char* what) { return strstr(name, what) != nullptr; }
+void set_basis(int* basis, int m, int n) {
+    for (int i = 0; i < m; ++i) basis[i] = i < fake_plan_k ? i : n + i;
+}
+void finish(DevState* st) {
+    st->status = fake_plan_status;
+    st->fail = fake_plan_fail;
+    st->iters = 7;
+}
+
+}  // namespace
+
+extern "C" void fake_play(const char* name, void** a) {
+    if (is(name, "k_reset_state")) {
+        DevState* st = *(DevState**)a[0];
+        memset(st, 0, sizeof *st);
+        st->status = tsx::kRunning;
+    } else if (is(name, "k_build")) {
+        set_basis(*(int**)a[8], *(int*)a[0], *(int*)a[1]);
+    } else if (is(name, "k_pivot_delayed") || is(name, "k_pivot_overlap")) {
+        finish(*(DevState**)a[3]);
+    } else if (is(name, "k_pivot_persistent") || is(name, "k_ml_update")) {
+        finish(((tsx::Params<double>*)a[0])->st);
+    } else if (is(name, "k_cluster_solve")) {
+        finish(((tsx::ClusterParams*)a[0])->st);
+    } else if (is(name, "k_team_solve")) {
+        auto* P = (tsx::TeamParams<double>*)a[0];
+        for (int l = 0; l < 2; ++l)
+            for (int k = 0; k < P->count[l]; ++k) {
+                const tsx::TeamJob<double>& J = P->jobs[P->order[l][k]];
+                set_basis(J.basis, J.m, J.n);
+                J.st->status = fake_plan_status;
+            }
+    } else if (is(name, "k_team_serve")) {
+        auto* P = (tsx::TeamServeParams<double>*)a[0];
+        for (unsigned l = 0; l < 2; ++l)
+            for (; P->head[l] != P->ring.tail[l]; ++P->head[l]) {
+                const unsigned slot = l * P->cap + (P->head[l] & (P->cap - 1u));
+                const tsx::TeamJob<double> J = P->ring.jobs[slot];
+                memset(J.st, 0, sizeof *J.st);
+                set_basis(J.basis, J.m, J.n);
+                J.st->status = fake_plan_status;
+                __atomic_store_n(P->ring.done + slot, P->head[l] + 1u, __ATOMIC_RELEASE);
+            }
+    }
+}

@@ -140,6 +140,22 @@ def test_overlapped_passes_time_out(tsx):   # noqa: F811
         np.testing.assert_array_equal(pr.tableau(), _oracle_run(A, b, c, max_iters=20).T)
 
 
+# limits around the length of a wait: a solve either times out or is right
+@pytest.mark.parametrize("m,n", [(300, 260), (1100, 1000)])
+def test_waits_that_run_out_late(tsx, m, n):   # noqa: F811
+    A, b, c = lpgen.dense_lp(m, n, 6)
+    ref = _oracle_run(A, b, c, max_iters=3)
+    with tsx.Problem(A, b, c) as pr:
+        for ns in list(range(600, 12000, 600)) * 10 + [10 ** 9]:
+            st = pr.solve(tsx.options(path=1, max_iters=3, barrier_timeout_ns=ns))
+            assert st == tsx.LP_ERR_TIMEOUT and ns < 10 ** 9 or st == tsx.LP_ITER_LIMIT
+            if st == tsx.LP_ITER_LIMIT:
+                sol = pr.solution()
+                assert sol.iters == 3 and sol.obj == ref.obj
+                np.testing.assert_array_equal(sol.x, ref.x)
+                np.testing.assert_array_equal(sol.y, ref.y)
+
+
 def test_many_with_a_large_lp(tsx):   # noqa: F811
     # an FP64 LP above 4e6 entries that would outlast its list is solved on the
     # whole grid
