@@ -322,8 +322,10 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(Tea
 //     that claimed a job just then kept the launch alive alone, and the stream
 //     behind it waited for that team: 7 s at 2000 LPs/s.)  Every wait is
 //     bounded: the claim loop by idle_cap_ns and a spin cap, after which the
-//     launch closes as well, the team barriers as in k_team_solve (a team that
-//     gives up clears its busy mark and closes the launch).
+//     launch closes as well, the other blocks' wait for their leader by more
+//     than that, the team barriers of a solve as in k_team_solve.  A team that
+//     gives up clears its busy mark, closes the launch and claims nothing more;
+//     an LP it has claimed is reported as timed out.
 // ---------------------------------------------------------------------------
 template <typename V>
 struct ServeRing {
@@ -367,10 +369,14 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
     TeamState* ts = P.tp.teams + t;
     const int li = P.tp.list[t];
     TeamJob<V>* jc = P.jcopy + t;
+    // the blocks of a team without work wait for their leader, which polls for
+    // up to idle_cap_ns, at a barrier (with timeout_ns alone, 2 s, they left a
+    // leader behind that then claimed an LP it could not solve)
+    const long long work_ns = P.idle_cap_ns + P.tp.timeout_ns;
     for (;;) {
+        int got = -1;   // the leader's: list of the LP it has claimed
         if (bt == 0 && threadIdx.x == 0) {
             ts->bad = 0;   // read after the next barrier; set during the build
-            int got = -1;
             unsigned gseq = 0;
             const long long t0 = global_ns();
             const unsigned long long max_spins =
@@ -378,6 +384,10 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
             long long t_idle = t0;   // since when no team has been seen working
             for (unsigned long long spins = 0;; ++spins) {
                 bool marked = false, closed = false;
+                if (ld_relaxed(&ts->fail) != 0) {   // a block of this team has left
+                    atomicOr(P.busy, kServeClosed);
+                    break;
+                }
                 for (int pass = 0; pass < 2 && got < 0 && !closed; ++pass) {
                     const int l = pass == 0 ? li : 1 - li;
                     const unsigned tl = ld_acquire_sys(P.ring.tail + l);
@@ -418,36 +428,40 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
                 for (int w = 0; w < (int)(sizeof(TeamJob<V>) / 8); ++w) dst[w] = src[w];
                 ts->job = (int)slot;
                 ts->seq = gseq;
+                // the LP's state words start from zero here (no reset launch per job)
+                DevState* st = jc->st;
+                st->status = kRunning;
+                st->q = -1;
+                st->p = -1;
+                st->bland = 0;
+                st->degen_run = 0;
+                st->bad = 0;
+                st->iters = 0;
+                st->active_sectors = 0;
+                st->theta = 0.0;
+                st->bar_count = 0;
+                st->bar_gen = 0;
+                st->nact = 0;
+                st->next_slot = 0;
+                st->fail = 0;
+                st->passes = 0;
+                for (int q = 2; q < 6; ++q) st->phase_ns[q] = 0;
+                st->phase_ns[1] = 0;
+                st->phase_ns[0] = global_ns();
             } else {
                 ts->job = -1;
             }
         }
-        if (!team_barrier(ts, C, P.tp.timeout_ns, s.ok, s.passed)) return;
+        if (!team_barrier(ts, C, work_ns, s.ok, s.passed)) {
+            if (bt == 0 && threadIdx.x == 0) {
+                atomicOr(P.busy, kServeClosed);
+                if (got >= 0) atomicSub(P.busy, 1u);
+            }
+            return;
+        }
         const int slot = *(volatile const int*)&ts->job;
         if (slot < 0) return;
         team_copy_job(s.job, jc);
-        if (bt == 0 && threadIdx.x == 0) {
-            // the LP's state words start from zero here (no reset launch per job)
-            DevState* st = s.job.st;
-            st->status = kRunning;
-            st->q = -1;
-            st->p = -1;
-            st->bland = 0;
-            st->degen_run = 0;
-            st->bad = 0;
-            st->iters = 0;
-            st->active_sectors = 0;
-            st->theta = 0.0;
-            st->bar_count = 0;
-            st->bar_gen = 0;
-            st->nact = 0;
-            st->next_slot = 0;
-            st->fail = 0;
-            st->passes = 0;
-            for (int q = 2; q < 6; ++q) st->phase_ns[q] = 0;
-            st->phase_ns[1] = 0;
-            st->phase_ns[0] = global_ns();
-        }
         if (!team_solve_one<NT>(P.tp, s.job, ts, bt, C, tsx_dyn, smem_bytes, s)) {
             if (bt == 0 && threadIdx.x == 0) {
                 atomicOr(P.busy, kServeClosed);

@@ -216,6 +216,33 @@ def test_bursts_around_the_idle_limit(tsx, pause):
     assert st["lane_lps"] == 240 and st["lane_launches"] >= (12 if pause >= 0.02 else 1)
 
 
+def test_a_team_that_has_waited_long_takes_a_request(tsx):
+    # one LP of several seconds keeps the team launch open; the other teams have
+    # then waited for work for longer than the limit of a barrier (2 s)
+    import torch
+    m = 10000
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    A = torch.rand(m, m, dtype=torch.float64, device="cuda", generator=g)
+    A.diagonal().add_(4.0 * m)
+    b = torch.rand(m, dtype=torch.float64, device="cuda", generator=g).mul_(900.0).add_(100.0)
+    c = torch.rand(m, dtype=torch.float64, device="cuda", generator=g).mul_(9.0).add_(1.0)
+    torch.cuda.synchronize()
+    A1, b1, c1 = lpgen.dense_lp(300, 260, 12)
+    alone = tsx.solve(A1, b1, c1)
+    with tsx.Server(precision=tsx.LP_PREC_FP64) as sv:
+        long = sv.submit_device(m, m, A, b, c)
+        time.sleep(2.3)
+        assert sv.wait(long, 0.0) == tsx.LP_PENDING
+        for _ in range(3):
+            t = sv.submit(A1, b1, c1)
+            assert sv.wait(t, 60.0) == tsx.LP_OPTIMAL, sv.last_error()
+            r = sv.result(t)
+            assert r.obj == alone.obj and r.iters == alone.iters
+            np.testing.assert_array_equal(r.x, alone.x)
+        assert sv.wait(long, 60.0) == tsx.LP_OPTIMAL
+
+
 @pytest.mark.parametrize("continuous", [1, 0])
 def test_invalid_device_request_in_a_wave(tsx, continuous):
     # device inputs are checked in the team kernel's build: a request with
