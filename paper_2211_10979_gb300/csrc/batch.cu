@@ -390,23 +390,22 @@ lp_batch_t lp_batch_create_device(int count, const int* m, const int* n, const d
     return h;
 }
 
-// The dynamic shared-memory limit of a kernel is process-wide state: it is
-// raised once per kernel instance to the device's maximum (never lowered, so
-// concurrent batches on other threads cannot race on it).
+// The dynamic shared-memory limit of a kernel is shared by a device's callers:
+// it is raised once per device and kernel instance to the device's maximum (never
+// lowered, so concurrent batches on other threads cannot race on it).
 template <int NT>
 static cudaError_t allow_max_smem() {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
+    static PerDevice<cudaError_t> done;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return done.get(dev, [dev] {
+        int optin = 0;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         cudaFuncAttributes fa{};
         cudaFuncGetAttributes(&fa, k_batch_solve<NT>);
-        err = cudaFuncSetAttribute(k_batch_solve<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   optin - (int)fa.sharedSizeBytes);
+        return cudaFuncSetAttribute(k_batch_solve<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    optin - (int)fa.sharedSizeBytes);
     });
-    return err;
 }
 
 template <int NT>

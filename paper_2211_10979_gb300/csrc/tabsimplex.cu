@@ -715,12 +715,15 @@ static const void* persistent_kernel(int m) {
 
 template <int NT, typename V>
 static void allow_persistent_smem() {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(persistent_kernel<NT, V>(1 << 30), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)persistent_smem<NT>());
-        cudaFuncSetAttribute(persistent_kernel<NT, V>(1), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)persistent_smem<NT>());
+    static PerDevice<cudaError_t> done;
+    int device = 0;
+    cudaGetDevice(&device);
+    done.get(device, [] {
+        const cudaError_t a = cudaFuncSetAttribute(persistent_kernel<NT, V>(1 << 30),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persistent_smem<NT>());
+        const cudaError_t b = cudaFuncSetAttribute(persistent_kernel<NT, V>(1),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persistent_smem<NT>());
+        return a != cudaSuccess ? a : b;
     });
 }
 
@@ -755,9 +758,9 @@ static size_t delayed_smem(int m, int n, int blocks, size_t limit) {
 template <int NT, typename V>
 static int delayed_coresident(int device, size_t& smem_limit) {
     constexpr int want = persistent_sm_threads(NT) / NT;   // blocks per SM the kernel is built for
-    static std::once_flag once;
-    static size_t limit = 0;
-    std::call_once(once, [device] {
+    static PerDevice<size_t> limits;
+    const size_t limit = limits.get(device, [device] {
+        size_t limit = 0;
         int per_sm = 0, reserved = 0, optin = 0;
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device);
@@ -771,6 +774,7 @@ static int delayed_coresident(int device, size_t& smem_limit) {
                 limit = (size_t)lim;
         }
         cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+        return limit;
     });
     smem_limit = limit;
     if (limit < delay_smem_bytes<V>(NT, kDelayedRows)) return 0;
@@ -832,10 +836,10 @@ static bool overlap_pays(int m, int n) {
 // (the passes then run in turn).  bytes: dynamic shared memory of a block.
 template <typename V>
 static int overlap_ready(lp_handle* h, const lp_options& o, int grid, size_t& bytes) {
-    static std::once_flag once;
-    static size_t limit = 0;
+    static PerDevice<size_t> limits;
     const int device = h->device;
-    std::call_once(once, [device] {
+    const size_t limit = limits.get(device, [device] {
+        size_t limit = 0;
         int optin = 0;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
         cudaFuncAttributes fa{};
@@ -844,6 +848,7 @@ static int overlap_ready(lp_handle* h, const lp_options& o, int grid, size_t& by
                                  optin - (int)fa.sharedSizeBytes) == cudaSuccess)
             limit = (size_t)optin - fa.sharedSizeBytes;
         cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+        return limit;
     });
     bytes = over_bytes<V>(h->m, h->n, grid);
     if (bytes > limit) return 0;
@@ -985,9 +990,14 @@ static size_t cluster_static_smem() {
 
 template <int NT>
 static cudaError_t cluster_allow(size_t smem) {
+    constexpr int kDevices = 64;
     static std::mutex mu;
-    static size_t allowed = 0;
+    static size_t allowed_on[kDevices] = {};   // per device, like the attributes
+    int device = 0;
+    cudaGetDevice(&device);
     std::lock_guard<std::mutex> lk(mu);
+    size_t beyond = 0;   // a device beyond the table: set at every call
+    size_t& allowed = device >= 0 && device < kDevices ? allowed_on[device] : beyond;
     if (smem <= allowed) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute((const void*)k_cluster_solve<NT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1444,7 +1454,7 @@ static lp_status ensure_recovery(lp_handle* h, int k) {
 }
 
 // Dynamic shared memory the LU kernels may use (raised to the device's limit
-// once); panel: whether the device can place the panel's cluster.
+// once per device); panel: whether the device can place the panel's cluster.
 struct LuLimits {
     size_t small_k = 0;
     bool panel = false;
@@ -1462,10 +1472,10 @@ static cudaLaunchConfig_t lu_panel_config(cudaStream_t s, cudaLaunchAttribute* a
     cfg.numAttrs = 1;
     return cfg;
 }
-static const LuLimits& lu_limits(int device) {
-    static std::once_flag once;
-    static LuLimits lim;
-    std::call_once(once, [device] {
+static LuLimits lu_limits(int device) {
+    static PerDevice<LuLimits> limits;
+    return limits.get(device, [device] {
+        LuLimits lim;
         int optin = 0;
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
         auto room = [&](const void* kernel) -> size_t {
@@ -1486,8 +1496,8 @@ static const LuLimits& lu_limits(int device) {
             cudaOccupancyMaxActiveClusters(&clusters, (const void*)k_lu_panel<256>, &cfg) == cudaSuccess && clusters > 0)
             lim.panel = true;
         cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+        return lim;
     });
-    return lim;
 }
 constexpr size_t kLuSharedSm = 100 * 1024;   // shared memory of the small kernel beside other work on its SM
 
@@ -1496,7 +1506,7 @@ constexpr size_t kLuSharedSm = 100 * 1024;   // shared memory of the small kerne
 // takes it.  blocks > 0: a share of the GPU beside other launches, one block.
 static lp_status recover_lu(lp_handle* h, const lp_options& o, cudaStream_t s, int k, long long& launches, bool& done) {
     RecBufs& r = h->rec;
-    const LuLimits& lim = lu_limits(h->device);
+    const LuLimits lim = lu_limits(h->device);
     const size_t cap = o.blocks > 0 ? std::min(lim.small_k, kLuSharedSm) : lim.small_k;
     done = true;
     if (k <= kLuSmallMax && lu_small_smem(k) <= cap) {
@@ -1590,9 +1600,9 @@ static lp_status recover_factor(lp_handle* h, const lp_options& o, cudaStream_t 
         long long to = std::max(0LL, o.barrier_timeout_ns);
         int kv = k;
         const size_t smem_ip = kk * 8 + bits;   // pivot row + used-row bitmap
-        static std::once_flag once;
-        static size_t ip_limit = 0;             // dynamic shared memory the in-place kernel may use
-        std::call_once(once, [optin] {
+        static PerDevice<size_t> limits;        // dynamic shared memory the in-place kernel may use
+        const size_t ip_limit = limits.get(h->device, [optin] {
+            size_t ip_limit = 0;
             cudaFuncAttributes fa{};
             if (cudaFuncGetAttributes(&fa, k_rec_gj_inplace<256>) == cudaSuccess &&
                 (size_t)optin > fa.sharedSizeBytes) {
@@ -1602,6 +1612,7 @@ static lp_status recover_factor(lp_handle* h, const lp_options& o, cudaStream_t 
                     ip_limit = lim;
             }
             cudaGetLastError();   // a refused attribute must not surface as a later launch's error
+            return ip_limit;
         });
         if (smem_ip <= ip_limit) {
             // in place on the k x k block (k_rec_gj_inplace)
@@ -1931,15 +1942,19 @@ lp_status lp_solve(lp_t h, const lp_options* opt) {
 
 // Dynamic shared memory that a block of a team kernel may use with as many
 // blocks per SM as the kernel is built for; the kernel's limit is raised to it
-// once (process-wide state, never lowered).
+// once per device (never lowered).
 template <int NT, typename V>
 static cudaError_t team_allow_smem(size_t& limit) {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    static size_t lim = 0;
-    std::call_once(once, [] {
-        int dev = 0, per_sm = 0, reserved = 0;
-        cudaGetDevice(&dev);
+    struct Limit {
+        size_t bytes = 0;
+        cudaError_t err = cudaSuccess;
+    };
+    static PerDevice<Limit> limits;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const Limit found = limits.get(dev, [dev] {
+        cudaError_t err = cudaSuccess;
+        int per_sm = 0, reserved = 0;
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
         constexpr int want = team_sm_threads(NT) / NT;
@@ -1950,12 +1965,13 @@ static cudaError_t team_allow_smem(size_t& limit) {
             if (err == cudaSuccess) err = cudaFuncGetAttributes(&fa, k);
             room = std::min(room, (long long)per_sm / want - reserved - (long long)fa.sharedSizeBytes);
         }
-        lim = (size_t)std::max(0LL, room / 128 * 128);
+        const size_t lim = (size_t)std::max(0LL, room / 128 * 128);
         for (const void* k : kernels)
             if (err == cudaSuccess) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
+        return Limit{lim, err};
     });
-    limit = lim;
-    return err;
+    limit = found.bytes;
+    return found.err;
 }
 
 // LPs whose pivot row would not fit one block's shared memory go to lp_solve,

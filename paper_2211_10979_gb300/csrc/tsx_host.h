@@ -5,6 +5,7 @@
 
 #include <cstddef>
 #include <functional>
+#include <mutex>
 #include <vector>
 
 #include "tabsimplex.h"
@@ -42,6 +43,24 @@ void stream_put(cudaStream_t s);
 // cudaHostRegister, torch's pinned tensors) that the current device may read
 // directly; null for pageable memory or memory not mapped for it.
 const double* host_alias(const double* p, size_t count);
+
+// One value per device, made on the first call for it (by whichever thread) and
+// kept: limits found while kernel attributes are raised, which belong to a
+// device and not to the process.  `make` runs with the device current.
+template <typename T>
+class PerDevice {
+    static constexpr int kMax = 64;
+    std::once_flag once_[kMax];
+    T value_[kMax]{};
+
+public:
+    template <typename Make>
+    T get(int device, Make make) {
+        if (device < 0 || device >= kMax) return make();
+        std::call_once(once_[device], [&] { value_[device] = make(); });
+        return value_[device];
+    }
+};
 
 struct DevState;
 // Uploads A (mn), b (m) and c (n) from their device aliases (host_alias) with

@@ -27,3 +27,36 @@ def test_a_block_that_gave_up_is_a_timeout(m, kernel):
     fake.fake_plan(0, 0, 0)
     assert solve({m}, {m}, path=1)[0] == tsx.LP_OPTIMAL
     """)
+
+
+def test_a_second_device_runs_the_same_kernels():
+    # kernel attributes (shared memory, cluster size) belong to a device
+    fakecuda.run("""
+    def calls(device):
+        fake.fake_reset()
+        fake.fake_plan(0, 0, 100)
+        st = [solve(300, 300, device, precision=tsx.LP_PREC_FP32)[0]]       # one-block LU, 86 KB
+        fake.fake_plan(0, 0, 400)
+        st.append(solve(500, 500, device, precision=tsx.LP_PREC_FP32)[0])   # panels: clusters of 16
+        fake.fake_plan(0, 0, 0)
+        for m, kw in ((256, {}), (600, {}), (300, {"path": 1}), (1000, {}), (300, {"threads": 128, "path": 1}),
+                      (300, {"layout": tsx.LP_LAYOUT_FULL})):
+            st.append(solve(m, m, device, **kw)[0])
+        for precision in (tsx.LP_PREC_FP64, tsx.LP_PREC_FP32):
+            prs = [tsx.Problem(*lp(300, 300)) for _ in range(3)]
+            st += tsx.solve_many(prs, tsx.options(precision=precision))
+            for pr in prs: pr.close()
+        with tsx.Batch([lp(120, 120)] * 3) as b:
+            b.solve(tsx.batch_options(threads=128))
+        assert set(st) == {tsx.LP_OPTIMAL}, (device, st, tsx.lp_last_error())
+        assert all(x[1] == device for x in log()), log()
+        return sorted((x[0],) + x[2:] for x in log())   # (recoveries run on several threads)
+    first = calls(0)
+    names = [x[0] for x in first]
+    for k in ("k_rec_lu_small", "k_lu_panel", "k_lu_solve", "k_cluster_solve", "k_pivot_delayed", "k_pivot_overlap",
+              "k_pivot_persistent", "k_team_solve", "k_batch_solve"):
+        assert k in names, (k, names)
+    for device in (1, 2, 70):   # 70: beyond the table of devices
+        assert calls(device) == first
+    assert calls(0) == first
+    """)
