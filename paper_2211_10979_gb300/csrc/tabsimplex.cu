@@ -1288,8 +1288,8 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     }
     // ... and the pass of a round may run behind the next round's pivots
     size_t osmem = 0;
-    const bool over = NT == 256 && dgrid > 0 && o.threads == 0 && overlap_pays<V>(m, n) &&
-                      overlap_ready<V>(h, o, dgrid, osmem) > 0;
+    bool over = NT == 256 && dgrid > 0 && o.threads == 0 && overlap_pays<V>(m, n) &&
+                overlap_ready<V>(h, o, dgrid, osmem) > 0;
     cudaEventRecord(h->ev[0], s);
     k_reset_state<<<1, 32, 0, s>>>(h->st);
     {
@@ -1351,16 +1351,21 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
                 Overlap<V> P2 = overlap_params<V>(h, D);
                 void* args2[] = {(void*)&P2, (void*)&eps_d, (void*)&eps_p, (void*)&st};
                 e = cudaLaunchCooperativeKernel((const void*)k_pivot_overlap<V>, dgrid, kOverNt, args2, osmem, s);
-                block_used = kOverNt;
-            } else {
-                e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
+                if (e == cudaSuccess) {
+                    block_used = kOverNt;
+                } else {   // refused: the passes in turn
+                    cudaGetLastError();
+                    over = false;
+                }
             }
+            if (!over)
+                e = cudaLaunchCooperativeKernel((const void*)k_pivot_delayed<NT, V>, dgrid, NT, args, dsmem, s);
         } else {
             e = launch_persistent<NT, V>(P, grid, s);
         }
         if (e != cudaSuccess) {
+            cudaGetLastError();             // must not surface as the next launch's error
             if (o.path == LP_PATH_AUTO) {   // co-residency refused: fall back
-                cudaGetLastError();
                 path = LP_PATH_MULTILAUNCH;
             } else {
                 set_error("lp_solve: cooperative launch failed: %s", cudaGetErrorString(e));

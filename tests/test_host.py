@@ -60,3 +60,23 @@ def test_a_second_device_runs_the_same_kernels():
         assert calls(device) == first
     assert calls(0) == first
     """)
+
+
+def test_a_refused_launch_takes_the_next_kernel():
+    fakecuda.run("""
+    fake.fake_refuse(b"k_pivot_overlap")
+    st, stats = solve(1000, 1000)
+    assert kernels()[-2:] == ["refused k_pivot_overlap", "k_pivot_delayed"], kernels()
+    assert st == tsx.LP_OPTIMAL and stats["path"] == tsx.LP_PATH_PERSISTENT and stats["block"] == 256
+    assert stats["update_bytes"] > 0
+    fake.fake_reset()
+    fake.fake_refuse(b"k_pivot_")   # none of them: one launch per phase
+    st, stats = solve(1000, 1000)
+    assert kernels()[4:7] == ["refused k_pivot_overlap", "refused k_pivot_delayed", "k_ml_init"], kernels()
+    assert st == tsx.LP_OPTIMAL and stats["path"] == tsx.LP_PATH_MULTILAUNCH and stats["block"] == 256
+    with tsx.Problem(*lp(1000, 1000)) as pr:
+        assert tsx.lp_solve(pr.h, tsx.options(path=tsx.LP_PATH_PERSISTENT)) == tsx.LP_ERR_CUDA
+        fake.fake_reset()
+        assert pr.solve(tsx.options(path=tsx.LP_PATH_PERSISTENT)) == tsx.LP_OPTIMAL
+        assert kernels()[-1] == "k_pivot_overlap" and pr.stats()["block"] == 512
+    """)
