@@ -199,6 +199,12 @@ def measured_peaks():
         return 6800.0, "fallback"
 
 
+def delayed_kernel(block, threads):
+    """The kernel of a condensed persistent solve: with the default threads only
+    the overlapped one has blocks of 512."""
+    return "k_pivot_overlap" if block == 512 and threads == 0 else "k_pivot_delayed"
+
+
 def profile_traffic(m, n, max_iters=-1, layout="condensed", grid=None, block=None):
     """ncu DRAM bytes per launch of the pivot kernel, if a summary for this
     exact kernel build and workload (FP64; a full solve, or the first
@@ -573,7 +579,7 @@ def run_gpu(args, rank, world, local):
             line["roofline"]["traffic"] = None
         delayed = stats[0]["path"] == 1 and args.layout == "condensed"
         if delayed:
-            line["roofline"]["kernel"] = "k_pivot_overlap" if stats[0]["block"] == 512 else "k_pivot_delayed"
+            line["roofline"]["kernel"] = delayed_kernel(stats[0]["block"], args.threads)
             line["roofline"]["what"] = ("bytes the pivots' update passes and side reads move (several pivots per "
                                         "pass over the tableau)")
         if delayed and args.precision == "fp64":

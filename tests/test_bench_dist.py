@@ -75,3 +75,10 @@ def test_truncated_fp32_solves_are_refused():
     with pytest.raises(SystemExit):
         bench.parse_args(["--precision", "fp32", "--max-iters", "5"])
     assert bench.parse_args(["--max-iters", "5"]).max_iters == 5
+
+
+def test_the_kernel_named_is_the_one_that_ran():
+    # --threads 512 runs k_pivot_delayed with blocks of 512
+    assert bench.delayed_kernel(512, 0) == "k_pivot_overlap"
+    assert bench.delayed_kernel(512, 512) == "k_pivot_delayed"
+    assert bench.delayed_kernel(256, 0) == bench.delayed_kernel(256, 256) == "k_pivot_delayed"
