@@ -88,6 +88,7 @@ struct Request {
     bool on_device = false;
     size_t bytes = 0;                     // device memory held while admitted
     bool small = false;
+    bool second_copy = false;             // bytes has room for a second copy of the tableau
     int status = 100;                     // running until done
     long long iters = 0;
     double obj = 0.0;
@@ -99,17 +100,14 @@ struct Request {
 };
 
 // Device bytes a request holds while it is solved: inputs, the condensed
-// tableau and work vectors, and for FP32 the FP64 recovery's k x 2k and k x k
-// matrices at their largest (k = min(m, n)).
+// tableau with its buffers, and for FP32 the FP64 recovery's k x 2k and k x k
+// matrices at their largest (k = min(m, n)); 1 MB for what does not grow with it.
 size_t request_bytes(int m, int n, bool small, int precision) {
     const size_t in = 8ull * ((size_t)m * n + m + n);
     if (small) return 2 * in + 8ull * (size_t)(m + 2) * (n + 3) + 64ull * (m + n) + 4096;
-    const size_t elem = precision == LP_PREC_FP32 ? 4 : 8;
-    const size_t ld = ((size_t)n + 1 + 31) / 32 * 32;
-    const size_t tab = (size_t)(m + 1) * ld * elem + (size_t)(m + 1 + 2 * ld) * elem;
     const size_t k = (size_t)std::min(m, n);
     const size_t rec = precision == LP_PREC_FP32 ? 24ull * k * k + 128ull * (m + n) : 0;
-    return in + tab + rec + 64ull * (m + n) + (1ull << 20);
+    return in + handle_bytes(m, n, precision) + rec + (1ull << 20);
 }
 
 }  // namespace
@@ -182,6 +180,7 @@ static void solve_single(lp_server* sv, Request& r, cudaStream_t s) {
         r.status = LP_ERR_INVALID;
         return;
     }
+    if (!r.second_copy) keep_one_copy(h);
     lp_options o;
     lp_options_init(&o);
     o.precision = sv->opt.precision;
@@ -308,6 +307,7 @@ static void solve_wave(lp_server* sv, std::vector<std::shared_ptr<Request>>& rs,
             r.status = LP_ERR_INVALID;
             continue;
         }
+        keep_one_copy(h);   // (an LP that no team takes is solved by lp_solve)
         hs.push_back(h);
         who.push_back(&r);
     }
@@ -683,6 +683,13 @@ static long long enqueue(lp_server* sv, std::shared_ptr<Request> r) {
     if ((long long)r->bytes > sv->opt.budget_bytes) {
         set_error("lps_submit: request needs %zu bytes, more than the budget", r->bytes);
         return -1;
+    }
+    // solved one at a time: with a second copy of the tableau if the budget has
+    // room for it
+    if (!r->small && sv->team_blocks < 0 && (sv->opt.path == LP_PATH_AUTO || sv->opt.path == LP_PATH_PERSISTENT)) {
+        const size_t more = second_copy_bytes(r->m, r->n, sv->opt.precision);
+        r->second_copy = more > 0 && (long long)(r->bytes + more) <= sv->opt.budget_bytes;
+        if (r->second_copy) r->bytes += more;
     }
     {
         std::lock_guard<std::mutex> lk(sv->mu);

@@ -155,6 +155,7 @@ struct lp_handle {
     int max_grid = 0;                // rpart capacity
     bool solved = false;
     bool checked = true;             // inputs validated (false: create_device_unchecked)
+    bool one_copy = false;           // never takes a second copy of the tableau (keep_one_copy)
     int last_status = LP_ERR_STATE;
     bool sol_ready = false;          // sol already holds the read-out (float path)
     std::vector<int> final_basis;    // float path: basic variables after the recovery
@@ -423,6 +424,25 @@ static bool ensure_events(lp_handle* h) {
     return true;
 }
 
+// Blocks whose partials a handle has room for (>= any co-resident grid).
+static int partial_capacity(int device) {
+    int nsm = 0;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+    return std::max(1, nsm) * 32;
+}
+
+// A handle's state block: state words, basis, read-out.
+struct CommonLayout {
+    size_t st, basis, sol, bytes;
+    CommonLayout(int m, int n) {
+        Carve cv;
+        st = cv.take(sizeof(DevState));
+        basis = cv.take((size_t)m * sizeof(int));
+        sol = cv.take((size_t)(n + m + 1) * sizeof(double));
+        bytes = align_up(cv.off, 256);
+    }
+};
+
 // Common part of the two create calls: sizes, stream, events, state block.
 static lp_handle* create_common(int m, int n, cudaStream_t stream, bool own_stream) {
     if (m <= 0 || n <= 0) {
@@ -455,22 +475,17 @@ static lp_handle* create_common(int m, int n, cudaStream_t stream, bool own_stre
         destroy_impl(h);
         return nullptr;
     }
-    int nsm = 0;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
-    h->max_grid = std::max(1, nsm) * 32;   // rpart capacity (>= any co-resident grid)
-    Carve cv;
-    const size_t o_st = cv.take(sizeof(DevState));
-    const size_t o_bs = cv.take((size_t)m * sizeof(int));
-    const size_t o_sol = cv.take((size_t)(n + m + 1) * sizeof(double));
-    if (!dev_alloc_block(h, h->common, align_up(cv.off, 256))) {
-        set_error("lp_create: device allocation of %zu bytes failed", cv.off);
+    h->max_grid = partial_capacity(h->device);
+    const CommonLayout at(m, n);
+    if (!dev_alloc_block(h, h->common, at.bytes)) {
+        set_error("lp_create: device allocation of %zu bytes failed", at.bytes);
         destroy_impl(h);
         return nullptr;
     }
     char* base = (char*)h->common.ptr;
-    h->st = (DevState*)(base + o_st);
-    h->basis = (int*)(base + o_bs);
-    h->sol = (double*)(base + o_sol);
+    h->st = (DevState*)(base + at.st);
+    h->basis = (int*)(base + at.basis);
+    h->sol = (double*)(base + at.sol);
     return h;
 }
 
@@ -638,52 +653,77 @@ lp_t lp_create_device(int m, int n, const double* dA, const double* db, const do
 // Leading dimension of a tableau of `elem`-byte entries: 128-byte rows.
 static int tableau_ld(int W, int elem) { return (int)align_up((size_t)W, 128 / elem); }
 
+// The pivot buffers of a tableau of `elem`-byte entries (cond: condensed).
+struct WorkLayout {
+    int Ws, ld;
+    size_t T, F, R, act, cpart, rpart, var, Fh, Rh, RhT, rhs, recs, bytes;
+    WorkLayout(int m, int n, int elem, int cond, int max_grid) {
+        Ws = cond ? n + 1 : n + m + 1;
+        ld = tableau_ld(Ws, elem);
+        const int E = 32 / elem;
+        const int nstrips = (ld + 32 * E - 1) / (32 * E);
+        const size_t K = cond ? (elem == 8 ? DelayK<double>::K : DelayK<float>::K) : 0;
+        Carve cv;
+        T = cv.take((size_t)(m + 1) * (size_t)ld * elem);
+        F = cv.take((size_t)(m + 1) * elem);
+        R = cv.take((size_t)ld * elem);
+        act = cv.take((size_t)(ld / E) * sizeof(int));
+        cpart = cv.take((size_t)nstrips * sizeof(ArgPart));
+        rpart = cv.take((size_t)max_grid * sizeof(RatPart));
+        var = cv.take((size_t)n * sizeof(int));
+        // the delayed updates'
+        Fh = cv.take((size_t)(m + 1) * K * elem);
+        Rh = cv.take((size_t)ld * K * elem);
+        RhT = cv.take((size_t)ld * K * elem);
+        rhs = cv.take(cond ? (size_t)(m + 1) * elem : 0);
+        recs = cv.take(cond ? 2 * (size_t)max_grid * sizeof(DelayRec) : 0);
+        bytes = align_up(cv.off, 256);
+    }
+};
+
+// A second copy of the condensed tableau and two rounds' buffers (overlapped
+// passes).
+struct CopyLayout {
+    size_t T, Fh, Rh, RhT, bytes;
+    CopyLayout(int m, int ld, size_t elem, size_t K) {
+        Carve cv;
+        T = cv.take((size_t)(m + 1) * (size_t)ld * elem);
+        Fh = cv.take(2 * (size_t)(m + 1) * K * elem);
+        Rh = cv.take(2 * (size_t)ld * K * elem);
+        RhT = cv.take(2 * (size_t)ld * K * elem);
+        bytes = align_up(cv.off, 256);
+    }
+};
+
 // (Re)allocates the pivot buffers for a tableau of `elem`-byte entries.
 static lp_status ensure_work(lp_handle* h, int elem, int cond) {
     if (h->work.elem == elem && h->work.cond == cond && h->work.blk.ptr) return LP_OPTIMAL;
     dev_free(h, h->work.blk);
     dev_free(h, h->work.blk2);
     h->work = Work{};
-    const int Ws = cond ? h->n + 1 : h->W;
-    const int ld = tableau_ld(Ws, elem);
-    const int E = 32 / elem;
-    const int nstrips = (ld + 32 * E - 1) / (32 * E);
-    Carve cv;
-    const size_t o_T = cv.take((size_t)(h->m + 1) * (size_t)ld * elem);
-    const size_t o_F = cv.take((size_t)(h->m + 1) * elem);
-    const size_t o_R = cv.take((size_t)ld * elem);
-    const size_t o_act = cv.take((size_t)(ld / E) * sizeof(int));
-    const size_t o_cp = cv.take((size_t)nstrips * sizeof(ArgPart));
-    const size_t o_rp = cv.take((size_t)h->max_grid * sizeof(RatPart));
-    const size_t o_var = cv.take((size_t)h->n * sizeof(int));
-    const size_t K = cond ? (elem == 8 ? DelayK<double>::K : DelayK<float>::K) : 0;
-    const size_t o_Fh = cv.take((size_t)(h->m + 1) * K * elem);
-    const size_t o_Rh = cv.take((size_t)ld * K * elem);
-    const size_t o_RhT = cv.take((size_t)ld * K * elem);
-    const size_t o_rhs = cv.take(cond ? (size_t)(h->m + 1) * elem : 0);
-    const size_t o_recs = cv.take(cond ? 2 * (size_t)h->max_grid * sizeof(DelayRec) : 0);
-    if (!dev_alloc_block(h, h->work.blk, align_up(cv.off, 256))) {
-        set_error("lp_solve: device allocation of %zu bytes for the tableau failed", cv.off);
+    const WorkLayout at(h->m, h->n, elem, cond, h->max_grid);
+    if (!dev_alloc_block(h, h->work.blk, at.bytes)) {
+        set_error("lp_solve: device allocation of %zu bytes for the tableau failed", at.bytes);
         return LP_ERR_NOMEM;
     }
     char* base = (char*)h->work.blk.ptr;
     h->work.elem = elem;
     h->work.cond = cond;
-    h->work.Ws = Ws;
-    h->work.ld = ld;
-    h->work.var = (int*)(base + o_var);
-    h->work.T = base + o_T;
-    h->work.F = base + o_F;
-    h->work.R = base + o_R;
-    h->work.act = (int*)(base + o_act);
-    h->work.cpart = (ArgPart*)(base + o_cp);
-    h->work.rpart = (RatPart*)(base + o_rp);
+    h->work.Ws = at.Ws;
+    h->work.ld = at.ld;
+    h->work.var = (int*)(base + at.var);
+    h->work.T = base + at.T;
+    h->work.F = base + at.F;
+    h->work.R = base + at.R;
+    h->work.act = (int*)(base + at.act);
+    h->work.cpart = (ArgPart*)(base + at.cpart);
+    h->work.rpart = (RatPart*)(base + at.rpart);
     if (cond) {
-        h->work.Fh = base + o_Fh;
-        h->work.Rh = base + o_Rh;
-        h->work.RhT = base + o_RhT;
-        h->work.rhs = base + o_rhs;
-        h->work.recs = (DelayRec*)(base + o_recs);
+        h->work.Fh = base + at.Fh;
+        h->work.Rh = base + at.Rh;
+        h->work.RhT = base + at.RhT;
+        h->work.rhs = base + at.rhs;
+        h->work.recs = (DelayRec*)(base + at.recs);
     }
     return LP_OPTIMAL;
 }
@@ -832,6 +872,21 @@ static bool overlap_pays(int m, int n) {
     return entries >= (sizeof(V) == 8 ? 1.0e6 : 2.2e7) && entries * sizeof(V) <= 4.3e9;
 }
 
+// (tsx_host.h) the account of a handle's buffers, from the layouts above
+size_t tsx::handle_bytes(int m, int n, int precision) {
+    int device = 0;
+    cudaGetDevice(&device);
+    const int elem = precision == LP_PREC_FP32 ? 4 : 8;
+    return CommonLayout(m, n).bytes + WorkLayout(m, n, elem, 1, partial_capacity(device)).bytes;
+}
+size_t tsx::second_copy_bytes(int m, int n, int precision) {
+    const bool fp32 = precision == LP_PREC_FP32;
+    if (!(fp32 ? overlap_pays<float>(m, n) : overlap_pays<double>(m, n))) return 0;
+    const size_t elem = fp32 ? 4 : 8;
+    return CopyLayout(m, tableau_ld(n + 1, (int)elem), elem, fp32 ? OverK<float>::K : OverK<double>::K).bytes;
+}
+void tsx::keep_one_copy(lp_t h) { h->one_copy = true; }
+
 // The grid and the second copy for overlapped passes; 0 where they do not fit
 // (the passes then run in turn).  bytes: dynamic shared memory of a block.
 template <typename V>
@@ -860,13 +915,8 @@ static int overlap_ready(lp_handle* h, const lp_options& o, int grid, size_t& by
         return 0;
     }
     if (!h->work.blk2.ptr) {
-        const size_t elem = sizeof(V), K = OverK<V>::K;
-        Carve cv;
-        cv.take((size_t)(h->m + 1) * (size_t)h->work.ld * elem);
-        cv.take(2 * (size_t)(h->m + 1) * K * elem);
-        cv.take(2 * (size_t)h->work.ld * K * elem);
-        cv.take(2 * (size_t)h->work.ld * K * elem);
-        if (!dev_alloc_block(h, h->work.blk2, align_up(cv.off, 256))) return 0;
+        const CopyLayout at(h->m, h->work.ld, sizeof(V), OverK<V>::K);
+        if (h->one_copy || !dev_alloc_block(h, h->work.blk2, at.bytes)) return 0;
         h->work.T2 = h->work.blk2.ptr;
     }
     return grid;
@@ -874,18 +924,13 @@ static int overlap_ready(lp_handle* h, const lp_options& o, int grid, size_t& by
 
 template <typename V>
 static Overlap<V> overlap_params(lp_handle* h, const Delayed<V>& D) {
-    const size_t elem = sizeof(V), K = OverK<V>::K;
-    Carve cv;
-    cv.take((size_t)(h->m + 1) * (size_t)h->work.ld * elem);
-    const size_t o_F = cv.take(2 * (size_t)(h->m + 1) * K * elem);
-    const size_t o_R = cv.take(2 * (size_t)h->work.ld * K * elem);
-    const size_t o_Rt = cv.take(2 * (size_t)h->work.ld * K * elem);
+    const CopyLayout at(h->m, h->work.ld, sizeof(V), OverK<V>::K);
     char* base = (char*)h->work.blk2.ptr;
     Overlap<V> P{};
     P.D = D;
-    P.D.Fh = (V*)(base + o_F);
-    P.D.Rh = (V*)(base + o_R);
-    P.D.RhT = (V*)(base + o_Rt);
+    P.D.Fh = (V*)(base + at.Fh);
+    P.D.Rh = (V*)(base + at.Rh);
+    P.D.RhT = (V*)(base + at.RhT);
     P.other = (V*)h->work.T2;
     return P;
 }
@@ -1428,7 +1473,7 @@ static lp_status ensure_recovery(lp_handle* h, int k) {
     }
     if (k > r.kcap) {
         dev_free(h, r.kb);
-        const int kc = std::max(std::max(k, 2 * std::max(r.kcap, 0)), 16);
+        const int kc = std::max(std::max(k, std::min(2 * std::max(r.kcap, 0), std::min(m, n))), 16);
         const size_t K = (size_t)kc;
         Carve cv;
         const size_t o_M = cv.take(K * 2 * K * 8), o_inv = cv.take(K * K * 8);

@@ -69,6 +69,14 @@ struct DevState;
 cudaError_t launch_ingest(const double* sA, double* dA, size_t mn, const double* sb, double* db, size_t m,
                           const double* sc, double* dc, size_t n, DevState* st, cudaStream_t s);
 
+// Device bytes that a handle allocates for a condensed solve in one copy of the
+// tableau, without its inputs and the FP64 recovery; and those of the second
+// copy that lp_solve adds on LP_PATH_AUTO and LP_PATH_PERSISTENT where the update
+// passes run behind the pivots (0: it adds none), unless keep_one_copy.
+size_t handle_bytes(int m, int n, int precision);
+size_t second_copy_bytes(int m, int n, int precision);
+void keep_one_copy(lp_t h);
+
 // Shared-memory bytes the batched solver has for one LP on the current device,
 // and whether an m x n LP fits in them.
 size_t batch_smem_limit();

@@ -80,3 +80,40 @@ def test_a_refused_launch_takes_the_next_kernel():
         assert pr.solve(tsx.options(path=tsx.LP_PATH_PERSISTENT)) == tsx.LP_OPTIMAL
         assert kernels()[-1] == "k_pivot_overlap" and pr.stats()["block"] == 512
     """)
+
+
+# what a request holds on the device against the server's account of it: long rows
+# (the delayed updates' buffers outweigh the vectors) and a tableau with a second
+# copy (passes behind the pivots), solved by the lane, by waves and one at a time
+@pytest.mark.parametrize("m,n,precision", [(16, 20000, 0), (16, 20000, 1), (20000, 16, 0), (1100, 1000, 0),
+                                           (300, 75000, 1)])
+@pytest.mark.parametrize("how", [{}, {"continuous": 0}, {"team_blocks": -1, "path": 0}, {"team_blocks": -1}])
+def test_a_request_holds_no_more_than_the_server_counts(m, n, precision, how):
+    fakecuda.run(f"""
+    import time
+    for k in (0, 16):
+        with tsx.Server(workers=1, batch_small=0, precision={precision}, **{how}) as sv:
+            fake.fake_reset()
+            fake.fake_plan(0, 0, k)
+            before = fake.fake_live()
+            t = sv.submit(*lp({m}, {n}))
+            assert sv.wait(t, 60.0) == tsx.LP_OPTIMAL, sv.last_error()
+            held, counted = fake.fake_peak() - before, sv.stats()["peak_bytes"]
+            assert 0 < held <= counted, (held, counted, kernels())
+    """)
+
+
+def test_a_budget_without_room_for_a_second_copy():
+    # still solved, in one copy of the tableau and within the budget
+    fakecuda.run("""
+    one, two = 20 << 20, 40 << 20
+    for budget, kernel in ((one, "k_pivot_delayed"), (two, "k_pivot_overlap")):
+        with tsx.Server(workers=1, batch_small=0, precision=tsx.LP_PREC_FP64, team_blocks=-1, path=0,
+                        budget_bytes=budget) as sv:
+            fake.fake_reset()
+            before = fake.fake_live()
+            t = sv.submit(*lp(1100, 1000))
+            assert sv.wait(t, 60.0) == tsx.LP_OPTIMAL, sv.last_error()
+            assert kernel in kernels(), kernels()
+            assert fake.fake_peak() - before <= sv.stats()["peak_bytes"] <= budget
+    """)
