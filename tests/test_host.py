@@ -117,3 +117,21 @@ def test_a_budget_without_room_for_a_second_copy():
             assert kernel in kernels(), kernels()
             assert fake.fake_peak() - before <= sv.stats()["peak_bytes"] <= budget
     """)
+
+
+def test_a_certain_cleanup_starts_from_the_inverse():
+    # after a capped or unbounded float phase the checks fail for certain, and the
+    # cleanup pivots need the explicit inverse: no LU before it
+    fakecuda.run("""
+    for status, inverse in ((tsx.LP_ITER_LIMIT, True), (tsx.LP_UNBOUNDED, True), (tsx.LP_OPTIMAL, False)):
+        for k, m in ((100, 300), (400, 500)):
+            fake.fake_reset()
+            fake.fake_plan(status, 0, k)
+            assert solve(m, m, precision=tsx.LP_PREC_FP32)[0] == tsx.LP_OPTIMAL
+            prs = [tsx.Problem(*lp(m, m)) for _ in range(2)]
+            assert tsx.solve_many(prs, tsx.options(precision=tsx.LP_PREC_FP32)) == [tsx.LP_OPTIMAL] * 2
+            for pr in prs: pr.close()
+            names = kernels()
+            assert ("k_rec_gj_inplace" in names) == inverse, (status, k, names)
+            assert any("_lu_" in x for x in names) != inverse, (status, k, names)
+    """)
