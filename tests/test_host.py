@@ -135,3 +135,14 @@ def test_a_certain_cleanup_starts_from_the_inverse():
             assert ("k_rec_gj_inplace" in names) == inverse, (status, k, names)
             assert any("_lu_" in x for x in names) != inverse, (status, k, names)
     """)
+
+
+# 700 x 500: a cluster block would hold more than 15000 entries, and the grid is
+# faster where it may use enough blocks
+@pytest.mark.parametrize("blocks,cluster", [(0, False), (1, True), (16, True), (63, True), (64, False), (152, False)])
+def test_a_capped_grid_does_not_take_a_clusters_place(blocks, cluster):
+    fakecuda.run(f"""
+    st, stats = solve(700, 500, blocks={blocks})
+    assert st == tsx.LP_OPTIMAL
+    assert stats["path"] == (tsx.LP_PATH_CLUSTER if {cluster} else tsx.LP_PATH_PERSISTENT), stats
+    """)
