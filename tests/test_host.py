@@ -146,3 +146,18 @@ def test_a_capped_grid_does_not_take_a_clusters_place(blocks, cluster):
     assert st == tsx.LP_OPTIMAL
     assert stats["path"] == (tsx.LP_PATH_CLUSTER if {cluster} else tsx.LP_PATH_PERSISTENT), stats
     """)
+
+
+# blocks of a delayed solve (152 SMs): as few as cost a solve alone next to
+# nothing, so that solves of several threads run side by side
+@pytest.mark.parametrize("m,n,precision,most,least", [
+    (300, 300, 0, 30, 24), (400, 400, 0, 50, 38), (512, 512, 0, 76, 64), (700, 500, 0, 76, 64), (700, 700, 0, 152, 152),
+    (1000, 1000, 0, 152, 152), (48, 48, 0, 13, 1), (256, 256, 1, 25, 8), (700, 700, 1, 30, 16), (1000, 1000, 1, 50, 32),
+    (1500, 1400, 1, 76, 64), (2000, 2000, 1, 152, 152), (3000, 100, 1, 50, 25), (33, 16384, 1, 152, 100)])
+def test_small_solves_leave_room_for_others(m, n, precision, most, least):
+    fakecuda.run(f"""
+    st, stats = solve({m}, {n}, precision={precision}, path=1)
+    assert st == tsx.LP_OPTIMAL and {least} <= stats["grid"] <= {most}, stats["grid"]
+    st, stats = solve({m}, {n}, precision={precision}, path=1, blocks=5)
+    assert stats["grid"] == 5
+    """)
