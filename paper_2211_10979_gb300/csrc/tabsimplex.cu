@@ -2299,6 +2299,8 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(base + o_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(base + o_next, 0, bytes - o_next, s);
+        const unsigned behind = (unsigned)nwide;   // each wide team starts with its own LP (k_team_solve)
+        if (e == cudaSuccess) e = cudaMemcpyAsync(P.next + 1, &behind, sizeof behind, cudaMemcpyHostToDevice, s);
         if (!ensure_events(h0)) return LP_ERR_CUDA;
         cudaEvent_t e0 = h0->ev[1], e1 = h0->ev[2];
         if (e == cudaSuccess) e = cudaEventRecord(e0, s);

@@ -62,7 +62,7 @@ struct TeamParams {
     const TeamJob<V>* jobs;
     const int* order[2];       // job indices of the two lists, largest first
     int count[2];              // their lengths
-    unsigned* next;            // list position counters (2)
+    unsigned* next;            // list position counters (2); [1] starts behind the wide teams' first LPs
     TeamState* teams;
     const int* team_of;        // grid: the team of each block
     const int* first;          // teams: first block, size, own list (0 or 1)
@@ -268,6 +268,10 @@ __device__ bool team_solve_one(const TeamParams<V>& P, const TeamJob<V>& J, Team
 
 // One cooperative launch: team t (blocks first[t] .. first[t] + size[t] - 1)
 // takes entries of its own list, then of the other one, until both are empty.
+// The wide teams, 0 .. their count - 1, start with that entry of their list: with
+// a counter alone a narrow team without work of its own could take an LP from a
+// wide team that began a moment later (5 FP64 LPs of 1000 x 900, blocks = 1: 55 ms
+// a call, 17 with every LP on a wide team).
 // Dynamic shared memory per block: smem_bytes, for the delayed solves.
 template <int NT, typename V>
 __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(TeamParams<V> P, unsigned smem_bytes) {
@@ -279,10 +283,10 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(Tea
     const unsigned C = (unsigned)P.size[t];
     TeamState* ts = P.teams + t;
     int li = P.list[t];
-    for (;;) {
+    for (bool start = true;; start = false) {
         if (bt == 0 && threadIdx.x == 0) {
             ts->bad = 0;   // read after the next barrier; set during the build
-            int k = -1;
+            int k = start && li == 1 ? P.order[1][t] : -1;
             for (int pass = 0; pass < 2 && k < 0; ++pass) {
                 const int l = pass == 0 ? li : 1 - li;
                 const int pos = (int)atomicAdd(P.next + l, 1u);

@@ -10,6 +10,8 @@
 
 extern "C" {
 int fake_plan_status = 0, fake_plan_fail = 0, fake_plan_k = 0;
+unsigned fake_team_next[2];   // k_team_solve: the list counters at its start
+int fake_team_wide = 0;       // and its wide teams
 }
 
 namespace {
@@ -41,6 +43,8 @@ extern "C" void fake_play(const char* name, void** a) {
         finish(((tsx::ClusterParams*)a[0])->st);
     } else if (is(name, "k_team_solve")) {
         auto* P = (tsx::TeamParams<double>*)a[0];
+        memcpy(fake_team_next, P->next, sizeof fake_team_next);
+        for (fake_team_wide = 0; P->first + fake_team_wide < P->size && P->list[fake_team_wide] == 1;) ++fake_team_wide;
         for (int l = 0; l < 2; ++l)
             for (int k = 0; k < P->count[l]; ++k) {
                 const tsx::TeamJob<double>& J = P->jobs[P->order[l][k]];

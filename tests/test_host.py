@@ -161,3 +161,16 @@ def test_small_solves_leave_room_for_others(m, n, precision, most, least):
     st, stats = solve({m}, {n}, precision={precision}, path=1, blocks=5)
     assert stats["grid"] == 5
     """)
+
+
+def test_wide_teams_start_with_their_own_lps():
+    # the heavy list's counter starts behind the wide teams' first LPs
+    fakecuda.run("""
+    for count, blocks in ((5, 1), (5, 2), (3, 0), (1, 0), (400, 1)):
+        prs = [tsx.Problem(*lp(100, 90 + 10 * (k < 3))) for k in range(count)]
+        assert tsx.solve_many(prs, tsx.options(blocks=blocks)) == [tsx.LP_OPTIMAL] * count
+        for pr in prs: pr.close()
+        nxt = list((ctypes.c_uint * 2).in_dll(fake, "fake_team_next"))
+        wide = ctypes.c_int.in_dll(fake, "fake_team_wide").value
+        assert nxt == [0, wide] and (wide > 0 or count == 400), (count, blocks, nxt, wide)
+    """)
