@@ -92,8 +92,8 @@ typedef struct {
                                      whole solve on chip, two cluster barriers
                                      per pivot) and has at most 600 rows and
                                      columns or less than 15000 entries per
-                                     block, or blocks is 1 to 63, else the
-                                     persistent
+                                     block, or `blocks` caps the grid, else
+                                     the persistent
                                      cooperative kernel when it can be
                                      launched, else one launch per phase;
                                      LP_PATH_PERSISTENT, LP_PATH_MULTILAUNCH or

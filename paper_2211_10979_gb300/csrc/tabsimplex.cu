@@ -1310,15 +1310,17 @@ static lp_status pivot_phase(lp_handle* h, const lp_options& o, cudaStream_t s, 
     // Tableau entries of a cluster block.  From 4000 on, 512 threads hide the
     // update's latencies better (us a pivot, 256 / 512 threads: 100^2 4.1 / 4.2,
     // 256^2 5.2 / 4.9, 400^2 8.3 / 6.8, 600^2 15.3 / 11.5).  From 15000 on the
-    // whole grid is faster (9.2 whatever the size up to 700^2), if it may use 64
-    // blocks (us a solve, cluster / grid of 32, 50, 64 blocks: 700x500 882 / 897,
-    // 819, 777; 1000x320 882 / 977, 886, 835; 500x700 620 / 636, 586, 551).  LPs
-    // up to 600 x 600 stay on the cluster although the grid would be faster from
-    // about 512^2 on: their path is the documented default.
+    // whole grid is faster (9.2 whatever the size up to 700^2; us a solve,
+    // cluster / grid: 700x500 882 / 768, 1000x320 882 / 821, 500x700 620 / 540).
+    // A capped grid leaves them on the cluster: on few blocks it is slower
+    // (700x500 with 32: 897), and a cap says that the device is shared, where a
+    // cluster's 16 SMs leave more room (8 threads solving 700x500: 264 / 403).
+    // LPs up to 600 x 600 stay on the cluster, although the grid would be faster
+    // from about 512^2 on: their path is the documented default.
     const long long centries = csize ? (long long)cluster_rows_per(m, csize) * (n + 1) : 0;
     const bool cwide = NT == 256 && o.threads == 0 && centries >= 4000;
-    if (path == LP_PATH_AUTO && std::max(m, n) > 600 && centries >= 15000 && (o.blocks <= 0 || o.blocks >= 64) &&
-        coop && coresident > 0)
+    if (path == LP_PATH_AUTO && std::max(m, n) > 600 && centries >= 15000 && coop && coresident > 0 &&
+        (o.blocks <= 0 || o.blocks >= coresident))
         csize = 0;
     if (path == LP_PATH_CLUSTER && !csize) {
         set_error("lp_solve: the cluster path needs an FP64 condensed tableau that fits one cluster's shared memory");

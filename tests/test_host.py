@@ -138,8 +138,8 @@ def test_a_certain_cleanup_starts_from_the_inverse():
 
 
 # 700 x 500: a cluster block would hold more than 15000 entries, and the grid is
-# faster where it may use enough blocks
-@pytest.mark.parametrize("blocks,cluster", [(0, False), (1, True), (16, True), (63, True), (64, False), (152, False)])
+# faster where it may use all of its blocks
+@pytest.mark.parametrize("blocks,cluster", [(0, False), (1, True), (16, True), (76, True), (151, True), (152, False)])
 def test_a_capped_grid_does_not_take_a_clusters_place(blocks, cluster):
     fakecuda.run(f"""
     st, stats = solve(700, 500, blocks={blocks})
