@@ -2571,6 +2571,8 @@ long long tsx::lane_submit(TeamLane* L, lp_t h) {
     L->pub[l] = seq + 1u;
     __atomic_store_n(L->tail_h + l, seq + 1u, __ATOMIC_RELEASE);
     L->out.push_back(TeamLane::Out{h, l, seq});
+    // (a launch that has not yielded yet keeps its SMs; one that has: lane_poll)
+    __atomic_store_n(L->stop_h, 0u, __ATOMIC_RELEASE);
     if (!L->running) {
         const lp_status st = L->fp32 ? lane_launch<float>(L) : lane_launch<double>(L);
         if (st != LP_OPTIMAL) return -1;
@@ -2620,6 +2622,11 @@ int tsx::lane_poll(TeamLane* L, std::vector<lp_t>& done) {
     return (int)L->out.size();
 }
 
+void tsx::lane_yield(TeamLane* L) {
+    std::lock_guard<std::mutex> lk(L->mu);
+    if (L->running && L->out.empty()) __atomic_store_n(L->stop_h, kServeYield, __ATOMIC_RELEASE);
+}
+
 lp_status tsx::lane_finish(TeamLane* L, lp_t h, cudaStream_t s, lp_status* status) {
     lp_options of = L->o;
     of.blocks = L->reserve;
@@ -2635,7 +2642,7 @@ long long tsx::lane_launches(TeamLane* L) {
 
 void tsx::lane_close(TeamLane* L) {
     if (!L) return;
-    if (L->stop_h) __atomic_store_n(L->stop_h, 1u, __ATOMIC_RELEASE);
+    if (L->stop_h) __atomic_store_n(L->stop_h, kServeStop, __ATOMIC_RELEASE);
     if (L->ks) cudaStreamSynchronize(L->ks);
     if (L->kev) cudaEventDestroy(L->kev);
     if (L->ks) cudaStreamDestroy(L->ks);

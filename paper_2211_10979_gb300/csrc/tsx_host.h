@@ -114,6 +114,9 @@ long long lane_submit(TeamLane* lane, lp_t h);
 // Returns the number of LPs still in the lane; waits on the device only to
 // read the claim counters after a launch has ended.
 int lane_poll(TeamLane* lane, std::vector<lp_t>& done);
+// Lets a launch that has no LP to solve end now instead of after its idle time
+// (for other work that needs its SMs).
+void lane_yield(TeamLane* lane);
 // Statistics and, for FP32, the FP64 recovery of a finished LP on stream s
 // (as lp_solve_many); *status receives its outcome.
 lp_status lane_finish(TeamLane* lane, lp_t h, cudaStream_t s, lp_status* status);

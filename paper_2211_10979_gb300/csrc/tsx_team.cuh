@@ -318,8 +318,9 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_solve(Tea
 //     system scope), which the host polls;
 //   - a team that finds nothing to claim keeps polling while another team
 //     still works (a job published meanwhile is taken at once); once no team
-//     has had work for idle_ns one of them closes the launch, every team exits,
-//     and the host starts a new launch when jobs are waiting and none runs.
+//     has had work for idle_ns (or at once, when the host asks for it) one of
+//     them closes the launch, every team exits, and the host starts a new launch
+//     when jobs are waiting and none runs.
 //     Closing is a bit of the busy word, set by a compare-and-swap from zero,
 //     and a team marks itself busy before it claims: a launch never goes on
 //     with some of its teams gone.  (When each team left on its own clock, one
@@ -336,7 +337,7 @@ struct ServeRing {
     TeamJob<V>* jobs;          // host memory: 2 lists x cap entries
     unsigned* tail;            // host memory: jobs published per list [2]
     unsigned* done;            // host memory: per entry, its sequence number + 1 once solved
-    unsigned* stop;            // host memory: nonzero: teams with nothing to claim exit now
+    unsigned* stop;            // host memory: kServeStop, kServeYield or 0
 };
 
 template <typename V>
@@ -352,6 +353,8 @@ struct TeamServeParams {
 };
 
 constexpr unsigned kServeClosed = 0x80000000u;   // no further job is claimed in this launch
+constexpr unsigned kServeStop = 1;    // teams with nothing to claim exit now
+constexpr unsigned kServeYield = 2;   // the launch closes as soon as no team works, without waiting for idle_ns
 
 __device__ __forceinline__ unsigned ld_acquire_sys(const unsigned* p) {
     unsigned v;
@@ -416,8 +419,10 @@ __global__ void __launch_bounds__(NT, team_sm_threads(NT) / NT) k_team_serve(Tea
                 const unsigned busy = *(volatile unsigned*)P.busy;
                 if (closed || (busy & kServeClosed)) break;
                 if (busy != 0u) t_idle = now;
-                if (ld_acquire_sys(P.ring.stop) != 0u) break;
-                if (now - t_idle >= P.idle_ns && atomicCAS(P.busy, 0u, kServeClosed) == 0u) break;
+                const unsigned stop = ld_acquire_sys(P.ring.stop);
+                if (stop == kServeStop) break;
+                if ((stop == kServeYield || now - t_idle >= P.idle_ns) && atomicCAS(P.busy, 0u, kServeClosed) == 0u)
+                    break;
                 if (now - t0 >= P.idle_cap_ns || spins >= max_spins) {
                     atomicOr(P.busy, kServeClosed);
                     break;

@@ -5,6 +5,7 @@
 // request.  Device memory is host memory; of the kernels only what the host
 // reads back is played (the state words, the final basis, the lane's rings).
 #include <cuda_runtime_api.h>
+#include <unistd.h>
 
 #include <cstdio>
 #include <cstdlib>
@@ -15,6 +16,7 @@
 
 // What a kernel leaves for the host to read (fake_kernels.cu).
 extern "C" void fake_play(const char* name, void** args);
+extern "C" int fake_lane_running();
 extern "C" int fake_plan_status, fake_plan_fail, fake_plan_k;   // what the next pivots end with
 
 namespace {
@@ -33,6 +35,12 @@ std::map<std::pair<int, const void*>, Attr> attrs;   // of (device, kernel)
 std::map<void*, size_t> blocks;                      // device allocations
 size_t live = 0, peak = 0;
 std::string log_text, refuse;
+// A lane's launch: the event recorded behind it is ready once it has ended, and
+// batch kernels launched meanwhile wait for that (fake_batch_waits).
+cudaEvent_t lane_event = nullptr;
+bool lane_launched = false;
+int batch_waits = 0;
+thread_local bool waits_for_lane = false;
 thread_local int device = 0;
 thread_local cudaError_t last = cudaSuccess;
 struct Call {
@@ -78,6 +86,8 @@ cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, size_t sme
         return fail(cudaErrorInvalidValue);
     }
     log_text += line;
+    if (is(name, "k_team_serve")) lane_launched = true;
+    if (is(name, "k_batch_solve") && batch_waits) waits_for_lane = true;
     fake_play(name.c_str(), args);
     return cudaSuccess;
 }
@@ -101,6 +111,7 @@ void fake_refuse(const char* what) { refuse = what; }
 const char* fake_log() { return log_text.c_str(); }
 long long fake_live() { return (long long)live; }
 long long fake_peak() { return (long long)peak; }
+void fake_batch_waits(int on) { batch_waits = on; }
 void fake_set_device(int d) { device = d; }
 
 // --------------------------------------------------------------- registration
@@ -262,7 +273,16 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {
     free(s);
     return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+    while (waits_for_lane) {
+        {
+            std::lock_guard<std::recursive_mutex> lk(mu);
+            waits_for_lane = fake_lane_running() != 0;
+        }
+        usleep(100);
+    }
+    return cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) {
     *st = cudaStreamCaptureStatusNone;
@@ -283,9 +303,19 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) {
     free(e);
     return cudaSuccess;
 }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) {
+    std::lock_guard<std::recursive_mutex> lk(mu);
+    if (lane_launched) {
+        lane_event = e;
+        lane_launched = false;
+    }
+    return cudaSuccess;
+}
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t e) {
+    std::lock_guard<std::recursive_mutex> lk(mu);
+    return e == lane_event && fake_lane_running() ? cudaErrorNotReady : cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {
     *ms = 1.f;
     return cudaSuccess;

@@ -2,6 +2,7 @@
 // basis and the lane's rings, from the library's own structs.
 #include <cuda_runtime.h>
 
+#include <chrono>
 #include <cstring>
 
 #include "tsx_cluster.cuh"
@@ -12,6 +13,7 @@ extern "C" {
 int fake_plan_status = 0, fake_plan_fail = 0, fake_plan_k = 0;
 unsigned fake_team_next[2];   // k_team_solve: the list counters at its start
 int fake_team_wide = 0;       // and its wide teams
+int fake_lane_ms = 0;         // the lane's launch stays for this long, or until its stop word is set
 }
 
 namespace {
@@ -19,6 +21,22 @@ using tsx::DevState;
 bool is(const char* name, const char* what) { return strstr(name, what) != nullptr; }
 void set_basis(int* basis, int m, int n) {
     for (int i = 0; i < m; ++i) basis[i] = i < fake_plan_k ? i : n + i;
+}
+// Solves what the rings hold.
+using Clock = std::chrono::steady_clock;
+tsx::TeamServeParams<double> lane;
+bool lane_open = false;
+Clock::time_point lane_end;
+void serve() {
+    for (unsigned l = 0; l < 2; ++l)
+        for (; lane.head[l] != __atomic_load_n(lane.ring.tail + l, __ATOMIC_ACQUIRE); ++lane.head[l]) {
+            const unsigned slot = l * lane.cap + (lane.head[l] & (lane.cap - 1u));
+            const tsx::TeamJob<double> J = lane.ring.jobs[slot];
+            memset(J.st, 0, sizeof *J.st);
+            set_basis(J.basis, J.m, J.n);
+            J.st->status = fake_plan_status;
+            __atomic_store_n(lane.ring.done + slot, lane.head[l] + 1u, __ATOMIC_RELEASE);
+        }
 }
 void finish(DevState* st) {
     st->status = fake_plan_status;
@@ -52,15 +70,17 @@ extern "C" void fake_play(const char* name, void** a) {
                 J.st->status = fake_plan_status;
             }
     } else if (is(name, "k_team_serve")) {
-        auto* P = (tsx::TeamServeParams<double>*)a[0];
-        for (unsigned l = 0; l < 2; ++l)
-            for (; P->head[l] != P->ring.tail[l]; ++P->head[l]) {
-                const unsigned slot = l * P->cap + (P->head[l] & (P->cap - 1u));
-                const tsx::TeamJob<double> J = P->ring.jobs[slot];
-                memset(J.st, 0, sizeof *J.st);
-                set_basis(J.basis, J.m, J.n);
-                J.st->status = fake_plan_status;
-                __atomic_store_n(P->ring.done + slot, P->head[l] + 1u, __ATOMIC_RELEASE);
-            }
+        lane = *(tsx::TeamServeParams<double>*)a[0];
+        lane_end = Clock::now() + std::chrono::milliseconds(fake_lane_ms);
+        lane_open = true;
+        serve();
     }
+}
+
+// Whether a lane's launch is on the device (called with the runtime's lock).
+extern "C" int fake_lane_running() {
+    if (!lane_open) return 0;
+    serve();
+    lane_open = Clock::now() < lane_end && __atomic_load_n(lane.ring.stop, __ATOMIC_ACQUIRE) == 0;
+    return lane_open;
 }

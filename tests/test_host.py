@@ -174,3 +174,29 @@ def test_wide_teams_start_with_their_own_lps():
         wide = ctypes.c_int.in_dll(fake, "fake_team_wide").value
         assert nxt == [0, wide] and (wide > 0 or count == 400), (count, blocks, nxt, wide)
     """)
+
+
+def test_an_idle_lane_makes_room_for_a_batch_that_waits_for_it():
+    # the lane's launch would stay for 3 s; a micro-batch whose blocks do not fit
+    # beside it is done long before, and later requests start a new launch
+    fakecuda.run("""
+    import time
+    lane_ms = ctypes.c_int.in_dll(fake, "fake_lane_ms")
+    lane_ms.value = 3000
+    with tsx.Server(workers=1, precision=tsx.LP_PREC_FP64) as sv:
+        def ask(m, n):
+            t = sv.submit(*lp(m, n))
+            t0 = time.perf_counter()
+            assert sv.wait(t, 60.0) == tsx.LP_OPTIMAL, sv.last_error()
+            sv.result(t)
+            return time.perf_counter() - t0
+        for launches in (1, 2, 3):
+            ask(300, 260)                       # the lane's
+            assert ask(64, 48) < 0.5            # a micro-batch beside it: the launch stays
+            assert ask(300, 260) < 0.5 and sv.stats()["lane_launches"] == launches
+            fake.fake_batch_waits(1)
+            assert ask(64, 48) < 0.5, launches
+            fake.fake_batch_waits(0)
+        lane_ms.value = 0
+        assert sv.stats()["batches"] == 6
+    """)
