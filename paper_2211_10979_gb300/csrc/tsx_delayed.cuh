@@ -377,9 +377,11 @@ __host__ __device__ constexpr size_t delay_smem_bytes(int nt, int rs) {
     return (size_t)kDelayStrips * DelayK<V>::K * 1024 + (size_t)(nt / 32) * DelayK<V>::K * (size_t)(rs * 8 + 16);
 }
 
-// 16-byte accesses, each of a warp's 512 contiguous bytes.  (256-bit ones of
-// four 64-bit words came back from ptxas 13.0 with the last three words not
-// updated in the builds with 128 registers a thread.)
+// 16-byte accesses, each of a warp's 512 contiguous bytes.  (With 256-bit ones of
+// four 64-bit words the team kernels' build, 128 registers a thread, gave wrong
+// tableaux: the last three words not updated, also with every word of the tile
+// set before its loads; k_pivot_delayed and k_pivot_overlap were right, and no
+// faster.  The cause is not known; nvcc 13.0.88.)
 __device__ __forceinline__ void ld_words(const void* p, unsigned long long* w) {
     asm volatile("ld.global.L1::no_allocate.v2.b64 {%0,%1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(p) : "memory");
 }
