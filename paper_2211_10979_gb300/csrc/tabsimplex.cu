@@ -854,19 +854,21 @@ static Delayed<V> delayed_params(lp_handle* h, const lp_options& o) {
 
 // Blocks of a delayed solve.  A pivot of a small LP is its chain of latencies,
 // whatever the grid, so it takes only the blocks that shorten it and solves of
-// other threads and streams run beside it: one block per 2800 entries (FP32:
-// 16000) or 100 rows or columns, at least 16 (at most one per four rows or
+// other threads and streams run beside it: one block per 2400 entries (FP32:
+// 16000) or 40 (80) rows or columns, at least 31 (at most one per four rows or
 // columns), rounded down to a whole fraction of the device's.  Measured, us a
 // solve alone on all blocks / on these, then with 8 threads solving: FP64 300^2
 // 420 / 422, 209 / 121; 512^2 636 / 633, 758 / 383; 700x500 756 / 768, 787 / 407;
-// FP32 512^2 716 / 706, 593 / 208; 1000^2 1188 / 1192, 1321 / 455; 1500x1400
-// 2230 / 2247, 1738 / 900.  Above, all blocks are faster: FP64 700^2 1332 / 1416
+// FP32 512^2 716 / 703, 593 / 210; 1000^2 1188 / 1192, 1321 / 455; 1500x1400
+// 2230 / 2247, 1738 / 900; with 15 or 21 blocks the smallest lose up to 7 % alone
+// (FP64 444x134 532 / 571, 549; 1069x42 227 / 239, 227), and FP64 4062x42 8 % with
+// 50 (760 / 829; 76 here).  Above, all blocks are faster: FP64 700^2 1332 / 1416
 // (76), FP32 2000^2 4612 / 4734.
 template <int NT, typename V>
 static int delayed_grid(int m, int n, int resident, int max_grid, int user_blocks) {
-    const double share = (sizeof(V) == 8 ? 2800.0 : 16000.0) * NT / 256.0;
-    const long long want = std::max<long long>(16, std::max<long long>((long long)((double)m * (double)n / share),
-                                                                       std::max(m, n) / 100));
+    const double share = (sizeof(V) == 8 ? 2400.0 : 16000.0) * NT / 256.0;
+    const long long want = std::max<long long>(31, std::max<long long>((long long)((double)m * (double)n / share),
+                                                                       std::max(m, n) / (sizeof(V) == 8 ? 40 : 80)));
     int g = std::max(1, resident);
     if (want < g) g /= (int)((g + want - 1) / want);
     g = std::min(std::min(g, max_grid), std::max(1, (std::max(m + 1, n) + 3) / 4));

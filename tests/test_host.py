@@ -152,7 +152,7 @@ def test_a_capped_grid_does_not_take_a_clusters_place(blocks, cluster):
 # nothing, so that solves of several threads run side by side
 @pytest.mark.parametrize("m,n,precision,most,least", [
     (300, 300, 0, 30, 24), (400, 400, 0, 50, 38), (512, 512, 0, 76, 64), (700, 500, 0, 76, 64), (700, 700, 0, 152, 152),
-    (1000, 1000, 0, 152, 152), (48, 48, 0, 13, 1), (256, 256, 1, 25, 8), (700, 700, 1, 30, 16), (1000, 1000, 1, 50, 32),
+    (1000, 1000, 0, 152, 152), (48, 48, 0, 13, 1), (256, 256, 1, 30, 24), (1069, 42, 0, 30, 24), (4062, 42, 0, 76, 64), (700, 700, 1, 30, 16), (1000, 1000, 1, 50, 32),
     (1500, 1400, 1, 76, 64), (2000, 2000, 1, 152, 152), (3000, 100, 1, 50, 25), (33, 16384, 1, 152, 100)])
 def test_small_solves_leave_room_for_others(m, n, precision, most, least):
     fakecuda.run(f"""
