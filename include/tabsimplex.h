@@ -113,8 +113,11 @@ typedef struct {
                                      0: update every column                     */
     int threads;                  /* threads per block, 0 = default (256; 512
                                      for large LPs and large cluster blocks)    */
-    int blocks;                   /* grid size cap, 0 = all co-resident blocks
-                                     (lp_solve_many: blocks per team)           */
+    int blocks;                   /* grid size cap, 0 = none: all co-resident
+                                     blocks for large LPs, fewer for small ones,
+                                     so that solves of other threads and streams
+                                     run beside them (lp_solve_many: blocks per
+                                     team)                                      */
     long long log_capacity;       /* pivots whose (q, p) pair is recorded;
                                      0 = none                                   */
     void *stream;                 /* cudaStream_t to run on; NULL = the
@@ -175,11 +178,20 @@ typedef struct {
                                      narrow team size)                          */
     int block;                    /* threads per block                          */
     int ld;                       /* leading dimension of the tableau (elems)   */
-    double phase_ms[6];           /* as seen by block 0.  Persistent path:
-                                     work time of {ratio test (Steps 1-2),
-                                     pivot-row staging, rank-1 update (Step
-                                     3)}, then the barrier wait after each of
-                                     them.  Cluster path: {Step 2, wait at
+    double phase_ms[6];           /* as seen by block 0.  Persistent path, full
+                                     layout: work time of {ratio test (Steps
+                                     1-2), pivot-row staging, rank-1 update
+                                     (Step 3)}, then the barrier wait after each
+                                     of them.  Condensed: {column q and its
+                                     ratios, row p and the objective row, the
+                                     update passes and the barrier before
+                                     each}, then the wait for the
+                                     leaving row, for the entering column and
+                                     after a pass; where the passes run behind
+                                     the pivots (512 threads), the third is the
+                                     wait for the running pass and the sixth
+                                     the end of a round (row and column stores
+                                     and their barriers).  Cluster path: {Step 2, wait at
                                      the first cluster barrier, cluster
                                      minimum and pivot-row slices, wait at the
                                      second cluster barrier, Step 3, Step 1}   */
@@ -231,7 +243,16 @@ lp_t lp_create_device(int m, int n, const double *dA, const double *db,
  * Steps 1-4 on one GPU) until termination.  Blocks until the device is done and
  * returns the termination status (>= 0) or an error (< 0).  May be called
  * again: every call starts over from the slack basis.  opt == NULL uses the
- * defaults. */
+ * defaults.
+ * Memory: the first solve allocates the tableau ((m+1) x ld entries, ld = n + 1
+ * condensed, rounded up to 128 bytes) and its work buffers, which the handle
+ * keeps until it solves in another precision or layout or is destroyed.  On the
+ * persistent path, condensed, with threads = 0, LPs of 1e6 entries (FP32:
+ * 2.2e7) or more and of up to 4.3 GB add a second copy of the tableau (and 16
+ * FP64 or 64 FP32 entries a row and twice that a column), for update passes that
+ * run behind the pivots; it stays with the handle too.  Where it cannot be
+ * allocated the solve goes on without it (the same results, up to a third
+ * slower); the allocator of lp_set_allocator sees that attempt. */
 lp_status lp_solve(lp_t h, const lp_options *opt);
 
 /* Solve `count` LPs at once, each from its slack basis (the method of
@@ -420,7 +441,9 @@ typedef struct lp_server *lps_t;
 
 typedef struct {
     long long budget_bytes;       /* device bytes admitted requests may hold
-                                     (tableau, inputs, work; default 64 GiB)    */
+                                     (tableau, inputs, work; a second copy of
+                                     the tableau only where there is room for
+                                     it; default 64 GiB)                        */
     int workers;                  /* concurrent solves (default 8)              */
     int precision;                /* single-LP lane (default LP_PREC_FP32)      */
     int batch_small;              /* 1 (default): micro-batch the small LPs     */
