@@ -260,9 +260,10 @@ lp_status lp_solve(lp_t h, const lp_options *opt);
  * launch divides the GPU into teams of opt->blocks thread blocks (default 16)
  * -- and, when some LPs carry more than a team's share of the list's work, up
  * to half of the GPU into wide teams of four times as many blocks that take
- * those LPs first; each team takes the next LP from its list, largest first
- * (then helps with the other list), and iterates on
- * its condensed tableau: block b of the team owns a contiguous range of rows
+ * those LPs first, and with blocks = 0 an FP64 list too short to fill the GPU
+ * gives every LP a team of its own; each team takes the next LP from its list,
+ * largest first (then helps with the other list), and iterates on its condensed
+ * tableau: block b of the team owns a contiguous range of rows
  * and of columns and brings its part of the entering column and of the pivot
  * row up to date, with two exchanges between the team's blocks per pivot; the
  * updates of up to 16 (FP32: 32) pivots share one pass over the tableau.  Meant

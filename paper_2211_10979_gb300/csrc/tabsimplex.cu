@@ -2150,6 +2150,39 @@ static lp_status finish_team_lp(lp_handle* h, const lp_options& o, cudaStream_t 
 #define TSX_TEAM_WIDE 1   // wide teams for the LPs heavier than a team's share
 #endif
 
+// Blocks of the LPs' own teams (FP64), `cap` together: the sizes at which the
+// slowest ends first, by an estimate of an LP's time (pivots ~ (m n)^0.62, each a
+// chain of latencies and its fused multiply-adds at a block's share of the pipe),
+// at least C and at most what a solve alone would take.
+template <int NT, typename V>
+static std::vector<int> own_team_sizes(const std::vector<lp_handle*>& hs, const std::vector<int>& who,
+                                       const std::vector<int>& order, int C, int cap, int nsm) {
+    const double chain = 9.0;     // us
+    const double rate = 2000.0;   // entries per us and block, two to an SM
+    auto sizes_for = [&](double us) {
+        std::vector<int> sizes;
+        for (int k : order) {
+            const lp_handle* h = hs[who[k]];
+            const double entries = (double)h->m * (double)h->n, per = us / std::pow(entries, 0.62) - chain;
+            const int most = std::min(kTeamMax, std::max(C, delayed_grid<NT, V>(h->m, h->n, nsm, h->max_grid, 0)));
+            const double want = per > 0.0 ? std::ceil(entries / (rate * per)) : most;
+            sizes.push_back((int)std::min<double>(most, std::max<double>(C, want)));
+        }
+        return sizes;
+    };
+    auto total = [](const std::vector<int>& sizes) {
+        int n = 0;
+        for (int s : sizes) n += s;
+        return n;
+    };
+    double lo = 0.0, hi = 1e12;   // (at hi every team has C blocks, which fit)
+    for (int i = 0; i < 80; ++i) {
+        const double mid = i < 40 ? std::sqrt(std::max(lo, 1.0) * hi) : 0.5 * (lo + hi);
+        (total(sizes_for(mid)) <= cap ? hi : lo) = mid;
+    }
+    return sizes_for(hi);
+}
+
 template <typename V>
 static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, cudaStream_t s,
                               lp_status* status, int reserve_blocks, const std::function<void()>& after_kernel) {
@@ -2232,24 +2265,34 @@ static lp_status solve_many_t(std::vector<lp_handle*>& hs, const lp_options& o, 
         const int CB = std::min(std::min(4 * C, kTeamMax), std::max(C, cap / 2));
         int nwide = heavy.empty() || CB <= C || !TSX_TEAM_WIDE ? 0
                                                                : std::min((int)heavy.size(), std::max(1, (cap / 2) / CB));
+        // An FP64 list whose teams of C would leave a quarter of the blocks or more
+        // idle: a team for each LP (us a call, one update per pivot -> delayed on
+        // teams of C and 4 C -> so: 8 x 1000^2 7670 -> 8380 -> 5100, 4 x 1000^2 6690 ->
+        // 8160 -> 3350; 29 lists of 2 to 14 LPs of 180 .. 3000 in geometric mean 1.12x
+        // of the second).  Not faster where less is idle (16 LPs 0.87x) nor in FP32,
+        // whose LPs are not bound by a team's pipes (1.00x).
+        const bool own_team = !fp32 && o.blocks == 0 && reserve_blocks == 0 && 4 * njobs * C <= 3 * cap;
+        if (own_team) {
+            heavy = order;
+            light.clear();
+            nwide = njobs;
+        }
         if (nwide == 0) {   // one list
             light.insert(light.begin(), heavy.begin(), heavy.end());
             heavy.clear();
         }
         std::vector<int> first, size, list, team_of;
-        for (int t = 0; t < nwide; ++t) {
+        auto add_team = [&](int blocks, int l) {
             first.push_back((int)team_of.size());
-            size.push_back(CB);
-            list.push_back(1);
-            team_of.insert(team_of.end(), CB, (int)first.size() - 1);
-        }
-        const int nnarrow = std::max(1, std::min((cap - nwide * CB) / C, njobs));
-        for (int t = 0; t < nnarrow && (int)team_of.size() + C <= cap; ++t) {
-            first.push_back((int)team_of.size());
-            size.push_back(C);
-            list.push_back(0);
-            team_of.insert(team_of.end(), C, (int)first.size() - 1);
-        }
+            size.push_back(blocks);
+            list.push_back(l);
+            team_of.insert(team_of.end(), blocks, (int)first.size() - 1);
+        };
+        if (own_team)
+            for (int s : own_team_sizes<NT, V>(hs, who, order, C, cap, nsm)) add_team(s, 1);
+        for (int t = 0; t < nwide && !own_team; ++t) add_team(CB, 1);
+        const int nnarrow = own_team ? 0 : std::max(1, std::min((cap - nwide * CB) / C, njobs));
+        for (int t = 0; t < nnarrow && (int)team_of.size() + C <= cap; ++t) add_team(C, 0);
         const int nteams = (int)first.size();
         const int grid = (int)team_of.size();
         // scratch: jobs | lists | counters | team tables | team states

@@ -13,6 +13,7 @@ extern "C" {
 int fake_plan_status = 0, fake_plan_fail = 0, fake_plan_k = 0;
 unsigned fake_team_next[2];   // k_team_solve: the list counters at its start
 int fake_team_wide = 0;       // and its wide teams
+int fake_team_size[512];      // blocks of each team (0: no such team)
 int fake_lane_ms = 0;         // the lane's launch stays for this long, or until its stop word is set
 }
 
@@ -62,6 +63,8 @@ extern "C" void fake_play(const char* name, void** a) {
     } else if (is(name, "k_team_solve")) {
         auto* P = (tsx::TeamParams<double>*)a[0];
         memcpy(fake_team_next, P->next, sizeof fake_team_next);
+        memset(fake_team_size, 0, sizeof fake_team_size);
+        for (int t = 0; t < 512 && P->first + t < P->size; ++t) fake_team_size[t] = P->size[t];
         for (fake_team_wide = 0; P->first + fake_team_wide < P->size && P->list[fake_team_wide] == 1;) ++fake_team_wide;
         for (int l = 0; l < 2; ++l)
             for (int k = 0; k < P->count[l]; ++k) {

@@ -200,3 +200,23 @@ def test_an_idle_lane_makes_room_for_a_batch_that_waits_for_it():
         lane_ms.value = 0
         assert sv.stats()["batches"] == 6
     """)
+
+
+def test_a_short_list_gives_every_lp_a_team():
+    fakecuda.run("""
+    def teams(shapes, **kw):
+        prs = [tsx.Problem(*lp(m, n)) for m, n in shapes]
+        assert tsx.solve_many(prs, tsx.options(**kw)) == [tsx.LP_OPTIMAL] * len(shapes)
+        for pr in prs: pr.close()
+        return [x for x in (ctypes.c_int * 512).in_dll(fake, "fake_team_size") if x]
+    assert teams([(1000, 1000)] * 8) == [38] * 8                       # 304 blocks
+    assert teams([(1000, 1000)] * 8, blocks=16) != [38] * 8            # the caller's team size
+    assert teams([(1000, 1000)] * 14) == [21] * 14
+    assert 64 in teams([(1000, 1000)] * 15)                            # little of the GPU is left
+    assert 64 in teams([(1000, 1000)] * 8, precision=tsx.LP_PREC_FP32)
+    assert teams([(200, 200)] * 2) == [30, 30]                         # more would not shorten them
+    mixed = teams([(300, 300), (1200, 1100), (600, 500)])              # largest first
+    assert mixed == sorted(mixed, reverse=True) and 16 <= mixed[2] and sum(mixed) <= 304 and mixed[0] > 100
+    assert sum(teams([(900 + 40 * k, 800) for k in range(11)])) <= 304
+    assert max(teams([(1400, 1400)])) <= 160
+    """)
